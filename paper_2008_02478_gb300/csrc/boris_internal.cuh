@@ -43,7 +43,8 @@ struct Geometry {
 // Launch schedule of the fused y-z spectral pass.
 struct YZSchedule {
     int kind;     // 0: fused, z stage through shared-memory passes; 1: fused, z stage in
-                  // registers; 2: split into y-forward, z-convolution and y-inverse kernels
+                  // registers; 2: split into y-forward, z-convolution and y-inverse kernels;
+                  // 3: the plane kernel on mixed-radix lengths (mixed_demag.cuh)
     int C;        // kinds 0/1: CTAs per cluster (one cluster per kx plane; ky residues mod C);
                   // kind 2: CTAs per SM targeted by the z-convolution's register budget
     int Qc;       // z-columns processed per chunk of the z stage
@@ -246,6 +247,8 @@ cudaError_t launch_curl_point(const Geometry& g, float2* Y, const float* KO, cud
 // Twiddle table exp(-2 pi i e / n), e in [0, n), on the host in FP64.
 void host_twiddles(int n, double2* out);
 
+struct MixedPlan;
+
 // Read-only view of a plan's geometry, schedule and kernel spectrum (capi.cu).
 struct PlanView {
     Geometry g;
@@ -257,6 +260,9 @@ struct PlanView {
     const void* tw;
     bool ml;       // multi-mesh plan
     bool oersted;  // Oersted plan: its spectrum is the curl kernel, not the demag tensor
+    const MixedPlan* mixed;  // mixed-radix path (schedule kind 3), else NULL
+    bool mixed_x1024;        // with the power-of-two x passes
+    size_t noalloc_need;     // its workspace need in boris_demag_apply_noalloc
 };
 // Number of kernel classes timed by the plan's profiler.
 constexpr int NPROF = 9;

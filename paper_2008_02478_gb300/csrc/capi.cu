@@ -14,6 +14,7 @@
 
 #include "boris_internal.cuh"
 #include "llg_kernels.cuh"
+#include "mixed_demag.cuh"
 #include "multilayer.cuh"
 
 using namespace boris;
@@ -77,6 +78,14 @@ struct boris_plan_s {
     double2* tw64 = nullptr;
     // spectral workspace [kx][c][z][y]
     void* X = nullptr;
+    // mixed-radix path (schedule kind 3): axis plans and their device tables; K
+    // then holds the spectrum [kx][kz'][pair][ky']
+    bool mixed = false;
+    MixedPlan mp = {};
+    bool mixed_x1024 = false;  // its x passes are the power-of-two ones (px 1024, 2048)
+    void* mtw = nullptr;
+    unsigned short* mpos = nullptr;
+    size_t noalloc_need = 0;  // bytes boris_demag_apply_noalloc asks for on this mesh
     // column-major padded spectrum [kx][ky][c][z] of the split schedule
     void* Y = nullptr;
     // LLG workspace (allocated on first use)
@@ -305,6 +314,15 @@ template <typename T>
 int demag_to_spectrum_t(boris_plan p, const T* M, const T* ms_map, T ms_scale)
 {
     using C = typename Cx<T>::t;
+    if (p->mixed) {
+        CUDA_TRY(timed(p, 0, [&] {
+            if (p->mixed_x1024)
+                return launch_x_r2c<T>(p->g, M, ms_map, ms_scale, (C*)p->X, (const C*)p->tw, p->stream);
+            return launch_mixed_x_fwd<T>(p->mp, M, ms_map, ms_scale, (C*)p->X, p->stream);
+        }));
+        CUDA_TRY(timed(p, 1, [&] { return launch_plane_conv<T>(p->mp, (C*)p->X, (const C*)p->K, p->stream); }));
+        return BORIS_OK;
+    }
     // FP16 spectrum: the x pass also finds max |Ms M| for the y passes' scale
     unsigned* absmax = nullptr;
     if constexpr (sizeof(T) == 4) {
@@ -338,6 +356,7 @@ int demag_apply_t(boris_plan p, const T* M, const T* ms_map, T ms_scale, T* H)
     int rc = demag_to_spectrum_t<T>(p, M, ms_map, ms_scale);
     if (rc) return rc;
     CUDA_TRY(timed(p, 2, [&] {
+        if (p->mixed && !p->mixed_x1024) return launch_mixed_x_inv<T>(p->mp, (const C*)p->X, H, p->stream);
         return launch_x_c2r<T>(p->g, (const C*)p->X, H, (const C*)p->tw, p->stream, p->d_status, p->wait_limit_ns);
     }));
     return BORIS_OK;
@@ -697,6 +716,42 @@ int llg_backward_t(boris_plan p, const T* m_in, const boris_llg_params* prm, dou
     return BORIS_OK;
 }
 
+// Uploads the tables of a mixed-radix plan and builds its kernel spectrum and workspace.
+int mixed_setup(boris_plan p)
+{
+    MixedPlan& m = p->mp;
+    const size_t esz = p->f64 ? sizeof(double2) : sizeof(float2);
+    size_t oy, oz;
+    const size_t n = mixed_tw_entries(m, &oy, &oz);
+    std::vector<double2> tw(n);
+    mixed_tw_fill(m, tw.data());
+    std::vector<float2> twf;
+    const void* src = tw.data();
+    if (!p->f64) {
+        for (const double2& v : tw) twf.push_back(make_float2((float)v.x, (float)v.y));
+        src = twf.data();
+    }
+    std::vector<unsigned short> pos(2 * (m.x.H + m.y.H));
+    line_pos_host(m.x, (int)esz, pos.data());
+    line_pos_host(m.y, (int)esz, pos.data() + 2 * m.x.H);
+    int rc;
+    CUDA_TRY(mixed_prepare(m, p->f64));
+    if ((rc = dev_alloc(p, &p->mtw, n * esz))) return rc;
+    if ((rc = dev_alloc(p, (void**)&p->mpos, pos.size() * sizeof(unsigned short)))) return rc;
+    CUDA_TRY(cudaMemcpy(p->mtw, src, n * esz, cudaMemcpyHostToDevice));
+    CUDA_TRY(cudaMemcpy(p->mpos, pos.data(), pos.size() * sizeof(unsigned short), cudaMemcpyHostToDevice));
+    m.twx = p->mtw;
+    m.twy = (const char*)p->mtw + oy * esz;
+    m.twz = (const char*)p->mtw + oz * esz;
+    m.posx = p->mpos;
+    m.posy = p->mpos + 2 * m.x.H;
+    if ((rc = dev_alloc(p, &p->K, mixed_kernel_entries(m) * esz))) return rc;
+    CUDA_TRY(build_mixed_spectrum(p->g, m, p->dx, p->dy, p->dz, 40.0, p->K, p->f64, p->stream, p->images));
+    if ((rc = dev_alloc(p, &p->X, (size_t)p->g.nkx * 3 * p->g.nz * p->g.ny * esz))) return rc;
+    CUDA_TRY(cudaStreamSynchronize(p->stream));
+    return BORIS_OK;
+}
+
 // Plan-time autotuner of the fused y-z pass: every candidate schedule that fits
 // the geometry runs on the (zeroed) spectral workspace, timed with CUDA events
 // on the plan's stream; the fastest is kept.
@@ -753,6 +808,9 @@ bool plan_view(boris_plan p, PlanView* v)
     v->tw = p->tw;
     v->ml = p->ml;
     v->oersted = p->oersted;
+    v->mixed = p->mixed ? &p->mp : nullptr;
+    v->mixed_x1024 = p->mixed_x1024;
+    v->noalloc_need = p->noalloc_need;
     return true;
 }
 }  // namespace boris
@@ -843,11 +901,49 @@ static int plan_create(int nx, int ny, int nz, double dx, double dy, double dz, 
     }
     int max_smem = 0;
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
+    // workspace of boris_demag_apply_noalloc on this mesh (power-of-two lengths)
+    const bool split_fits = p->f64 ? split_supported<double>(g, max_smem) : split_supported<float>(g, max_smem);
+    p->noalloc_need = (((size_t)g.nkx * 3 * nz * ny * sizeof(float2) + 255) & ~(size_t)255) +
+                      (split_fits ? (size_t)g.nkx * g.py * 3 * nz * sizeof(float2) : 0);
+    // Mixed-radix lengths with the whole kx plane in one CTA's shared memory,
+    // where they pay (mixed_pays) and no switch pins another schedule;
+    // BORIS_YZ_KIND=3 takes them wherever the plane fits.
+    const char* kind = std::getenv("BORIS_YZ_KIND");
+    const bool forced = kind && std::atoi(kind) == 3;
+    bool pinned = tc != 0 || (kind && !forced);
+    for (const char* v : {"BORIS_YZ_CLUSTER", "BORIS_YZ_THREADS", "BORIS_YZ_QC", "BORIS_YZ_TMA"})
+        pinned |= std::getenv(v) != nullptr;
+    if (const char* sf = std::getenv("BORIS_FUSE_STAGE")) pinned |= std::atoi(sf) == 1;
+    if (!pinned && mixed_plan_shape(nx, ny, nz, p->f64, max_smem, &p->mp) && (forced || mixed_pays(p->mp, p->f64, g))) {
+        p->mixed = true;
+        Geometry& mg = p->g;
+        mg.px = 2 * p->mp.x.H;
+        mg.py = 2 * p->mp.y.H;
+        mg.pz = nz == 1 ? 1 : 2 * p->mp.HZ;
+        mg.nkx = p->mp.x.H + 1;
+        mg.kyh = p->mp.y.H + 1;
+        mg.kzh = p->mp.nkz;
+        // x rows of 1024 or 2048 padded values: the warp-held transforms, one trip
+        // through shared memory instead of three, win once there are enough rows for
+        // their 16- and 8-row tiles (512 x 512 x 1: 5.2 against 7.1 us a pass, 512 x 512
+        // x 8: 20 against 29; 1024 x 1024 x 2: 29 against 33)
+        p->mixed_x1024 = !p->f64 && (mg.px == 1024 || mg.px == 2048) && (long)ny * nz >= 256;
+        if (p->mixed_x1024) {
+            mg.lgx = ilog2(mg.px);
+            mg.lmax = mg.px;
+            mg.lglmax = mg.lgx;
+            if ((rc = upload_plan_twiddles(p, mg, false))) return bail(rc);
+        }
+        p->yz = YZSchedule{3, 1, 0, p->mp.threads, p->mp.smem};
+        if ((rc = mixed_setup(p))) return bail(rc);
+        *out = p;
+        return BORIS_OK;
+    }
     YZSchedule cand[20];
     int ncand = 0;
     if (p->f64) yz_candidates<double>(g, max_smem, cand, &ncand);
     else yz_candidates<float>(g, max_smem, cand, &ncand);
-    const bool split_ok = p->f64 ? split_supported<double>(g, max_smem) : split_supported<float>(g, max_smem);
+    const bool split_ok = split_fits;
     if (split_ok && ncand < 14) {
         cand[ncand++] = YZSchedule{2, 2, 0, 0, 0};
         if (!p->f64) cand[ncand++] = YZSchedule{2, 3, 0, 0, 0};
@@ -1642,7 +1738,7 @@ void boris_plan_destroy(boris_plan p)
 {
     if (!p) return;
     cudaStreamSynchronize(p->stream);
-    void* ptrs[] = {p->d_absmax, p->Y16, p->K16, p->Kml, p->d_pairs, p->d_pcode, p->d_invhz, p->Mf, p->Hf, p->K, p->K2, p->d_step, p->X, p->Y, p->Hd, p->msa, p->msb, p->acc, p->kbuf, p->mtrial, p->d_rkf, p->energy,
+    void* ptrs[] = {p->mtw, p->mpos, p->d_absmax, p->Y16, p->K16, p->Kml, p->d_pairs, p->d_pcode, p->d_invhz, p->Mf, p->Hf, p->K, p->K2, p->d_step, p->X, p->Y, p->Hd, p->msa, p->msb, p->acc, p->kbuf, p->mtrial, p->d_rkf, p->energy,
                     p->m_dev_e2e, p->bw};
     for (void* q : ptrs)
         if (q) cudaFree(q);

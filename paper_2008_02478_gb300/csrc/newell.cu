@@ -19,7 +19,11 @@
 //    store -Re / (px py pz) as rows [kx][ky] of kz * 6 + component (row
 //    length padded to a multiple of 4 with zeros) in FP32 or FP64.
 #include "boris_internal.cuh"
+#include "mixed_demag.cuh"
 #include "newell_fg.cuh"
+
+#include <algorithm>
+#include <vector>
 
 namespace boris {
 
@@ -300,6 +304,173 @@ cudaError_t build_kernel_spectrum(const Geometry& g, double dx, double dy, doubl
     if (T) cudaFreeAsync(T, st);
     if (A) cudaFreeAsync(A, st);
     if (B) cudaFreeAsync(B, st);
+    return e;
+}
+
+// ---------------------------------------------------------------------------
+// The same spectrum on mixed-radix lengths (mixed_fft.cuh): one axis pass per
+// axis in FP64, the octant line extended to length 2 H by its parity and
+// folded into the two half-length inputs e[n] = x[n] + x[n + H] (even bins)
+// and o[n] = x[n] - x[n + H] (odd bins) while it is loaded; bins 0..H kept.
+// ---------------------------------------------------------------------------
+template <typename L>
+__global__ void __launch_bounds__(256) mixed_axis_kernel(const void* __restrict__ in, bool in_real,
+                                                         double2* __restrict__ out, int axis, int d0, int d1, int d2,
+                                                         int NL, const double2* __restrict__ tw,
+                                                         const unsigned short* __restrict__ pos)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double2* buf = reinterpret_cast<double2*>(smem_raw);  // [NL][LS]
+    const int dims[3] = {d0, d1, d2};
+    int od[3] = {d0, d1, d2};
+    constexpr int H = L::H, kh = H + 1;
+    const int n = dims[axis];
+    od[axis] = kh;
+    const int oa = axis == 0 ? 1 : 0, ob = axis == 2 ? 1 : 2;
+    const long total = 6L * dims[oa] * dims[ob];
+    const long line0 = (long)blockIdx.x * NL;
+    const int nl = (int)min((long)NL, total - line0);
+    // line -> component and the base offset of its entry 0 in an array of extents e[]
+    auto base_of = [&](long line, const int* e, int& c) -> size_t {
+        int co[3] = {0, 0, 0};
+        co[oa] = (int)(line % dims[oa]);
+        const long rest = line / dims[oa];
+        co[ob] = (int)(rest % dims[ob]);
+        c = (int)(rest / dims[ob]);
+        return (size_t)c * e[0] * e[1] * e[2] + ((size_t)co[2] * e[1] + co[1]) * e[0] + co[0];
+    };
+    const size_t is = axis == 0 ? 1 : axis == 1 ? d0 : (size_t)d0 * d1;
+    const size_t os = axis == 0 ? 1 : axis == 1 ? od[0] : (size_t)od[0] * od[1];
+    line_fwd1<L, true>(nl, buf, tw, [&](int l, int i, bool par) {
+        int c;
+        const size_t b = base_of(line0 + l, dims, c);
+        auto at = [&](int e) {  // entry e of the extended line, 0 <= e < 2 H
+            double2 v = make_double2(0.0, 0.0);
+            const int src = e < n ? e : e > 2 * H - n ? 2 * H - e : -1;
+            if (src >= 0) {
+                const double s = e < n ? 1.0 : comp_parity(c, axis);
+                if (in_real) v.x = s * reinterpret_cast<const double*>(in)[b + src * is];
+                else {
+                    const double2 t = reinterpret_cast<const double2*>(in)[b + src * is];
+                    v = make_double2(s * t.x, s * t.y);
+                }
+            }
+            return v;
+        };
+        const double2 u = at(i), w = at(i + H);
+        return par ? c_sub(u, w) : c_add(u, w);
+    });
+    line_fwd_rest<L>(nl, buf, tw);
+    for (int i = threadIdx.x; i < nl * kh; i += blockDim.x) {
+        const int l = i / kh, k = i % kh;
+        int c;
+        const size_t b = base_of(line0 + l, od, c);
+        out[b + k * os] = buf[l * L::template LS<double2> + pos[k]];
+    }
+}
+
+// K[kx][kz'][pair][ky'], pairs (xx, yy), (zz, xy), (xz, yz); entries past ky' = H are zero
+template <typename T>
+__global__ void mixed_finalize_kernel(const double2* __restrict__ S, typename Cx<T>::t* __restrict__ K, int nkx, int kyh,
+                                      int kzh, int kyp, double scale)
+{
+    const size_t n = (size_t)nkx * kyh * kzh, total = (size_t)nkx * kzh * 3 * kyp;
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+        const int ky = (int)(i % kyp);
+        size_t row = i / kyp;
+        const int pair = (int)(row % 3);
+        row /= 3;
+        const int kz = (int)(row % kzh), kx = (int)(row / kzh);
+        typename Cx<T>::t v{T(0), T(0)};
+        if (ky < kyh) {
+            // components xx yy zz xy xz yz
+            const int c0 = pair == 0 ? 0 : pair == 1 ? 2 : 4, c1 = pair == 0 ? 1 : pair == 1 ? 3 : 5;
+            const size_t at = ((size_t)kz * kyh + ky) * nkx + kx;
+            v.x = (T)(-S[c0 * n + at].x * scale);
+            v.y = (T)(-S[c1 * n + at].x * scale);
+        }
+        K[i] = v;
+    }
+}
+
+cudaError_t build_mixed_spectrum(const Geometry& g, const MixedPlan& m, double dx, double dy, double dz, double rs,
+                                 void* K, bool f64, cudaStream_t st, const int* images)
+{
+    const int nn[3] = {g.nx, g.ny, g.nz};
+    LineFFT f[3];
+    std::vector<double2> tw;
+    std::vector<unsigned short> pos;
+    size_t two[3] = {}, poso[3] = {};
+    for (int a = 0; a < 3; a++) {
+        if (nn[a] < 2) continue;
+        // the padded lengths of the plan: the z axis has its own list of half lengths
+        const int H = a == 0 ? m.x.H : a == 1 ? m.y.H : m.HZ;
+        if (!make_line_fft(H, (int)sizeof(double2), false, &f[a]) || f[a].H != H) return cudaErrorInvalidValue;
+        two[a] = tw.size();
+        tw.resize(tw.size() + line_tw_entries(f[a]));
+        line_tw_host(f[a], tw.data() + two[a]);
+        poso[a] = pos.size();
+        pos.resize(pos.size() + 2 * H);
+        line_pos_host(f[a], (int)sizeof(double2), pos.data() + poso[a]);
+    }
+    const size_t n = (size_t)g.nx * g.ny * g.nz;
+    const int dims[4][3] = {{g.nx, g.ny, g.nz}, {g.nkx, g.ny, g.nz}, {g.nkx, g.kyh, g.nz}, {g.nkx, g.kyh, g.kzh}};
+    auto elems = [&](int i) { return 6 * (size_t)dims[i][0] * dims[i][1] * dims[i][2]; };
+    void* cur = nullptr;  // the octant, then the spectrum after each axis
+    double2* dtw = nullptr;
+    unsigned short* dpos = nullptr;
+    cudaError_t e = cudaMallocAsync(&cur, 6 * n * sizeof(double), st);
+    if (e == cudaSuccess) e = cudaMallocAsync((void**)&dtw, (tw.size() + 1) * sizeof(double2), st);
+    if (e == cudaSuccess) e = cudaMallocAsync((void**)&dpos, (pos.size() + 1) * sizeof(unsigned short), st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dtw, tw.data(), tw.size() * sizeof(double2), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(dpos, pos.data(), pos.size() * sizeof(unsigned short), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // the host tables end with this call
+    if (e == cudaSuccess) e = newell_octant(g.nx, g.ny, g.nz, dx, dy, dz, rs, (double*)cur, st, images);
+    bool real = true;
+    for (int a = 0; a < 3 && e == cudaSuccess; a++) {
+        if (nn[a] < 2) continue;
+        void* next = nullptr;
+        if ((e = cudaMallocAsync(&next, elems(a + 1) * sizeof(double2), st)) != cudaSuccess) break;
+        int NL = 1;
+        while (NL < 16 && (size_t)2 * NL * f[a].LS * sizeof(double2) <= 72 * 1024) NL *= 2;
+        const size_t smem = (size_t)NL * f[a].LS * sizeof(double2);
+        const int oa = a == 0 ? 1 : 0, ob = a == 2 ? 1 : 2;
+        const long lines = 6L * dims[a][oa] * dims[a][ob];
+        const unsigned blocks = (unsigned)((lines + NL - 1) / NL);
+        switch (f[a].id) {
+#define X(i, r1, r2, r3, ...)                                                                                              \
+    case i:                                                                                                           \
+        e = cudaFuncSetAttribute(mixed_axis_kernel<Len<r1, r2, r3, __VA_ARGS__>>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
+                                 96 * 1024);                                                                          \
+        if (e == cudaSuccess)                                                                                         \
+            mixed_axis_kernel<Len<r1, r2, r3, __VA_ARGS__>><<<blocks, 256, smem, st>>>(cur, real, (double2*)next, a, dims[a][0],   \
+                                                                          dims[a][1], dims[a][2], NL, dtw + two[a],   \
+                                                                          dpos + poso[a]);                            \
+        break;
+            BORIS_LENGTHS_FINE(X)
+#undef X
+        }
+        if (e == cudaSuccess) e = cudaGetLastError();
+        cudaFreeAsync(cur, st);
+        cur = next;
+        real = false;
+    }
+    if (e == cudaSuccess) {
+        const double scale = 1.0 / ((double)g.px * g.py * g.pz);
+        const size_t tot = mixed_kernel_entries(m);
+        const int blocks = (int)std::min<size_t>((tot + 255) / 256, 152 * 64);
+        if (f64)
+            mixed_finalize_kernel<double><<<blocks, 256, 0, st>>>((const double2*)cur, (double2*)K, g.nkx, g.kyh, g.kzh,
+                                                                  m.kyp, scale);
+        else
+            mixed_finalize_kernel<float><<<blocks, 256, 0, st>>>((const double2*)cur, (float2*)K, g.nkx, g.kyh, g.kzh,
+                                                                 m.kyp, scale);
+        e = cudaGetLastError();
+    }
+    if (cur) cudaFreeAsync(cur, st);
+    if (dtw) cudaFreeAsync(dtw, st);
+    if (dpos) cudaFreeAsync(dpos, st);
     return e;
 }
 

@@ -19,6 +19,7 @@
 #include <string>
 
 #include "boris_internal.cuh"
+#include "mixed_demag.cuh"
 
 namespace boris {
 
@@ -77,7 +78,7 @@ extern "C" int boris_demag_apply_noalloc(boris_plan p, const float* M, float* Hd
     // the split y-z schedule also needs the column-major padded spectrum
     const size_t ybytes = v.yz.kind == 2 ? (size_t)v.g.nkx * v.g.py * 3 * v.g.nz * sizeof(float2) : 0;
     const size_t xoff = (xbytes + 255) & ~(size_t)255;
-    const size_t need = xoff + ybytes;
+    const size_t need = v.mixed ? v.noalloc_need : xoff + ybytes;
     if (need > NOALLOC_SCRATCH_BYTES) {
         set_error("mesh spectrum needs " + std::to_string(need) + " bytes; the allocation-free workspace holds " +
                   std::to_string(NOALLOC_SCRATCH_BYTES) + " bytes (use boris_demag_apply)");
@@ -96,6 +97,19 @@ extern "C" int boris_demag_apply_noalloc(boris_plan p, const float* M, float* Hd
     // clearing between calls
     const float2* tw = (const float2*)v.tw;
     float2* Y = (float2*)((unsigned char*)X + xoff);
+    if (v.mixed) {
+        e = v.mixed_x1024 ? launch_x_r2c<float>(v.g, M, nullptr, 1.0f, X, tw, v.stream)
+                          : launch_mixed_x_fwd<float>(*v.mixed, M, nullptr, 1.0f, X, v.stream);
+        if (e == cudaSuccess) e = launch_plane_conv<float>(*v.mixed, X, (const float2*)v.K, v.stream);
+        if (e == cudaSuccess)
+            e = v.mixed_x1024 ? launch_x_c2r<float>(v.g, X, Hd, tw, v.stream)
+                              : launch_mixed_x_inv<float>(*v.mixed, X, Hd, v.stream);
+        if (e != cudaSuccess) {
+            set_error(std::string("demag kernels: ") + cudaGetErrorString(e));
+            return BORIS_ERR_CUDA;
+        }
+        return BORIS_OK;
+    }
     if ((e = launch_x_r2c<float>(v.g, M, nullptr, 1.0f, X, tw, v.stream)) == cudaSuccess) {
         if (v.yz.kind == 2) {
             for (int part = 0; part < 3 && e == cudaSuccess; part++)
