@@ -380,6 +380,7 @@ int check_params(boris_plan p, const boris_llg_params* prm, LLGArgs<T>* a, doubl
     a->ihy2 = (T)(1.0 / (p->dy * p->dy));
     a->ihz2 = (T)(1.0 / (p->dz * p->dz));
     a->Ms = (T)prm->Ms;
+    a->inv_ms = T(1) / ((T)MU0_D * a->Ms);
     a->Ku = (T)prm->Ku;
     a->A = (T)prm->A;
     a->ms_map = (const T*)prm->Ms_map;
@@ -412,6 +413,9 @@ int check_params(boris_plan p, const boris_llg_params* prm, LLGArgs<T>* a, doubl
     a->hx = (T)p->dx;
     a->hy = (T)p->dy;
     a->hz = (T)p->dz;
+    a->i2hx = T(0.5) / a->hx;
+    a->i2hy = T(0.5) / a->hy;
+    a->i2hz = T(0.5) / a->hz;
     a->J1 = (T)t.J1;
     a->J2 = (T)t.J2;
     a->pbc = p->pbc;
@@ -419,6 +423,7 @@ int check_params(boris_plan p, const boris_llg_params* prm, LLGArgs<T>* a, doubl
     a->th_s0 = (T)((p->has_terms && t.temperature > 0 && dt > 0)
                        ? std::sqrt(2.0 * prm->alpha * kB * t.temperature / (prm->gamma * MU0_D * a->V * dt))
                        : 0.0);
+    a->th_sg = a->th_s0 / std::sqrt(a->Ms);
     a->seed_lo = (unsigned int)(t.seed & 0xffffffffull);
     a->seed_hi = (unsigned int)(t.seed >> 32);
     a->step = p->d_step;
@@ -514,8 +519,8 @@ int rkf45_trial_t(boris_plan p, const T* m, LLGArgs<T> a)
     return BORIS_OK;
 }
 
-// The CUDA graph of one RKF45 step: begin (no trial yet) -> WHILE(trial,
-// controller) -> accept (m = trial if accepted).  The controller ends the loop
+// The CUDA graph of one RKF45 step: WHILE(trial, controller) -> accept (m =
+// trial if accepted).  The controller ends the loop
 // when a trial is accepted or RKF_MAX_TRIALS were rejected, so one launch of
 // the graph never runs more than RKF_MAX_TRIALS trials and needs no host
 // decision.
@@ -540,8 +545,7 @@ int rkf45_graph_t(boris_plan p, T* m, const boris_llg_params* prm, const LLGArgs
     p->prof = false;
     int rc = BORIS_OK;
     cudaError_t e = cudaSuccess;
-    cudaGraphNode_t begin = nullptr, loop = nullptr;
-    size_t nn = 0;
+    cudaGraphNode_t loop = nullptr;
     cudaGraphConditionalHandle cond = 0;
     auto capture_into = [&](cudaGraph_t target, const cudaGraphNode_t* dep, size_t ndep, auto&& body) -> cudaError_t {
         cudaError_t ce = cudaStreamBeginCaptureToGraph(p->gstream, target, dep, nullptr, ndep,
@@ -552,14 +556,7 @@ int rkf45_graph_t(boris_plan p, T* m, const boris_llg_params* prm, const LLGArgs
         cudaError_t ce2 = cudaStreamEndCapture(p->gstream, &out);
         return ce2;
     };
-    // 1. begin
-    e = capture_into(g, nullptr, 0, [&] {
-        cudaError_t le = launch_rkf45_begin(p->d_rkf, p->gstream);
-        if (le != cudaSuccess) rc = fail(BORIS_ERR_CUDA, std::string("rkf45 begin: ") + cudaGetErrorString(le));
-    });
-    if (e == cudaSuccess && rc == BORIS_OK) e = cudaGraphGetNodes(g, nullptr, &nn);
-    if (e == cudaSuccess && rc == BORIS_OK && nn == 1) e = cudaGraphGetNodes(g, &begin, &nn);
-    // 2. the trial loop
+    // 1. the trial loop
     if (e == cudaSuccess && rc == BORIS_OK) e = cudaGraphConditionalHandleCreate(&cond, g, 1u, cudaGraphCondAssignDefault);
     cudaGraph_t body = nullptr;
     if (e == cudaSuccess && rc == BORIS_OK) {
@@ -568,7 +565,7 @@ int rkf45_graph_t(boris_plan p, T* m, const boris_llg_params* prm, const LLGArgs
         np.conditional.handle = cond;
         np.conditional.type = cudaGraphCondTypeWhile;
         np.conditional.size = 1;
-        e = cudaGraphAddNode(&loop, g, &begin, nullptr, 1, &np);
+        e = cudaGraphAddNode(&loop, g, nullptr, nullptr, 0, &np);
         if (e == cudaSuccess) body = np.conditional.phGraph_out[0];
     }
     long long trial_launches = 0;
@@ -585,7 +582,7 @@ int rkf45_graph_t(boris_plan p, T* m, const boris_llg_params* prm, const LLGArgs
         });
         trial_launches = p->launches - b0;
     }
-    // 3. accept
+    // 2. accept
     if (e == cudaSuccess && rc == BORIS_OK) {
         e = capture_into(g, &loop, 1, [&] {
             cudaError_t le = launch_rkf45_accept<T>(p->d_rkf, (const T*)p->mtrial, m, 3 * ncell(p), p->gstream);
@@ -633,7 +630,7 @@ int rkf45_run_t(boris_plan p, T* m, const boris_llg_params* prm, double* dt, int
     CUDA_TRY(cudaMemcpyAsync(p->h_rkf, p->d_rkf, sizeof(RKFControl), cudaMemcpyDeviceToHost, p->stream));
     CUDA_TRY(cudaStreamSynchronize(p->stream));
     const RKFControl& c = *p->h_rkf;
-    p->launches += 1 + (long long)nsteps * 2 + (long long)c.trials * p->rkf_trial_launches;
+    p->launches += 1 + (long long)nsteps + (long long)c.trials * p->rkf_trial_launches;
     *dt = c.dt;
     if (t_elapsed) *t_elapsed = c.t;
     if (c.failed_steps > 0)

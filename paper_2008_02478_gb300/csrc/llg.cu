@@ -18,33 +18,32 @@
 
 namespace boris {
 
-// Runge-Kutta-Fehlberg 4(5) coefficients (Fehlberg's published tableau):
-// stage s state = m0 + dt sum_j A[s][j] k_j; 4th/5th order weights B4, B5.
-__constant__ double RKF_A[6][5] = {
-    {0, 0, 0, 0, 0},
-    {1.0 / 4, 0, 0, 0, 0},
-    {3.0 / 32, 9.0 / 32, 0, 0, 0},
-    {1932.0 / 2197, -7200.0 / 2197, 7296.0 / 2197, 0, 0},
-    {439.0 / 216, -8.0, 3680.0 / 513, -845.0 / 4104, 0},
-    {-8.0 / 27, 2.0, -3544.0 / 2565, 1859.0 / 4104, -11.0 / 40},
-};
-__constant__ double RKF_B4[6] = {25.0 / 216, 0.0, 1408.0 / 2565, 2197.0 / 4104, -1.0 / 5, 0.0};
-__constant__ double RKF_B5[6] = {16.0 / 135, 0.0, 6656.0 / 12825, 28561.0 / 56430, -9.0 / 50, 2.0 / 55};
-
-// stage s in 0..3; ms = stage state (m0 itself for s = 0).
-template <typename T>
-__global__ void __launch_bounds__(256) rk4_stage_kernel(LLGArgs<T> a, int s, const T* __restrict__ ms,
+// Stage S in 0..3; ms = stage state (m0 itself for S = 0).  What the update
+// reads of the cell is loaded with the stencil, not behind the field: the
+// kernel is bound by load latency on small meshes (101 x 100 x 3 4.4 -> 2.6 us,
+// 512 x 512 x 1 with DMI and thermal field 9.3 -> 8 us) and by its instructions
+// with the further terms (512 x 512 x 32 256 -> 178 us); FP64 by the FP64 units
+// (128 x 128 x 16 63 -> 41 us with the uniform 1/(mu0 Ms) from the host).
+template <typename T, bool EXTRA, int S>
+__global__ void __launch_bounds__(256) rk4_stage_kernel(LLGArgs<T> a, const T* __restrict__ ms,
                                                         const T* __restrict__ Hd, T* __restrict__ m0,
                                                         T* __restrict__ acc, T* __restrict__ mnext)
 {
-    const size_t n = a.ncell;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % a.nx);
-        const int y = (int)((i / a.nx) % a.ny);
-        const int z = (int)(i / ((size_t)a.nx * a.ny));
+    const unsigned n = (unsigned)a.ncell, nx = a.nx, ny = a.ny;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const unsigned row = i / nx;
+        const int x = (int)(i - row * nx), z = (int)(row / ny), y = (int)(row - (unsigned)z * ny);
+        T b[3] = {}, ac[3] = {};
+        if (S > 0) {
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                b[c] = m0[c * n + i];
+                ac[c] = acc[c * n + i];
+            }
+        }
         T m[3], k[3];
-        field_and_rhs(a, ms, Hd, i, x, y, z, m, k);
-        rk4_combine(a, s, i, m, k, m0, acc, mnext);
+        field_and_rhs<EXTRA>(a, ms, Hd, i, x, y, z, m, k);
+        rk4_combine(a, S, i, m, k, b, ac, m0, acc, mnext);
     }
 }
 
@@ -180,57 +179,36 @@ __global__ void __launch_bounds__(256, 4) rk4_stage_quad_kernel(LLGArgs<float> a
     }
 }
 
-// RKF45 stage s in 0..5: k_s = f(ms); for s < 5 writes the next stage state
-// mnext = m0 + dt sum_{j<=s} a_{s+1,j} k_j; for s = 5 writes the normalised
-// 4th-order solution into mnext and folds max |m5 - m4| into *err.
-template <typename T>
-__global__ void __launch_bounds__(256) rkf45_stage_kernel(LLGArgs<T> a, int s, const T* __restrict__ ms,
+// RKF45 stage S in 0..5: k_S = f(ms); for S < 5 writes the next stage state
+// mnext = m0 + dt sum_{j<=S} a_{S+1,j} k_j; for S = 5 writes the normalised
+// 4th-order solution into mnext and folds max |m5 - m4| into *err.  The stage is
+// a template argument so that the earlier rates load at once (256 x 64 x 1
+// 5.3 -> 2.5 us, 512 x 512 x 32 520 -> 110..250 us a stage).
+template <typename T, bool EXTRA, int S>
+__global__ void __launch_bounds__(256) rkf45_stage_kernel(LLGArgs<T> a, const T* __restrict__ ms,
                                                           const T* __restrict__ Hd, const T* __restrict__ m0,
                                                           T* __restrict__ kbuf, T* __restrict__ mnext,
                                                           unsigned long long* __restrict__ err_bits)
 {
-    const size_t n = a.ncell;
+    const unsigned n = (unsigned)a.ncell, nx = a.nx, ny = a.ny;
     const T dt = a.dt_dev ? (T)*a.dt_dev : a.dt;
     double local_err = 0.0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % a.nx);
-        const int y = (int)((i / a.nx) % a.ny);
-        const int z = (int)(i / ((size_t)a.nx * a.ny));
-        T m[3], k[3];
-        field_and_rhs(a, ms, Hd, i, x, y, z, m, k);
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const unsigned row = i / nx;
+        const int x = (int)(i - row * nx), z = (int)(row / ny), y = (int)(row - (unsigned)z * ny);
+        // what the combination reads is loaded with the stencil, not behind it
+        T b[3], kj[3][S > 0 ? S : 1];
 #pragma unroll
-        for (int c = 0; c < 3; c++) kbuf[((size_t)s * 3 + c) * n + i] = k[c];
-        if (s < 5) {
+        for (int c = 0; c < 3; c++) {
+            b[c] = m0[c * n + i];
 #pragma unroll
-            for (int c = 0; c < 3; c++) {
-                T v = m0[c * n + i];
-                for (int j = 0; j < s; j++) v += dt * T(RKF_A[s + 1][j]) * kbuf[((size_t)j * 3 + c) * n + i];
-                v += dt * T(RKF_A[s + 1][s]) * k[c];
-                mnext[c * n + i] = v;
-            }
-        } else {
-            T v4[3];
-            double e2 = 0.0;
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                T s4 = T(0);
-                double d = 0.0;  // m5 - m4 = dt sum_j (b5_j - b4_j) k_j, accumulated in FP64
-                for (int j = 0; j < 6; j++) {
-                    const T kj = j == 5 ? k[c] : kbuf[((size_t)j * 3 + c) * n + i];
-                    s4 += T(RKF_B4[j]) * kj;
-                    d += (RKF_B5[j] - RKF_B4[j]) * (double)kj;
-                }
-                v4[c] = m0[c * n + i] + dt * s4;
-                d *= (double)dt;
-                e2 += d * d;
-            }
-            local_err = fmax(local_err, sqrt(e2));
-            const T inv = T(1) / sqrt(v4[0] * v4[0] + v4[1] * v4[1] + v4[2] * v4[2]);
-#pragma unroll
-            for (int c = 0; c < 3; c++) mnext[c * n + i] = v4[c] * inv;
+            for (int j = 0; j < S; j++) kj[c][j] = kbuf[(size_t)(j * 3 + c) * n + i];
         }
+        T m[3], k[3];
+        field_and_rhs<EXTRA>(a, ms, Hd, i, x, y, z, m, k);
+        rkf45_update<S>(n, i, k, dt, b, kj, kbuf, mnext, local_err);
     }
-    if (s == 5) {
+    if (S == 5) {
         // non-negative doubles order like their bit patterns read as unsigned integers
         for (int o = 16; o > 0; o >>= 1) local_err = fmax(local_err, __shfl_xor_sync(0xffffffffu, local_err, o));
         if ((threadIdx.x & 31) == 0) atomicMax(err_bits, (unsigned long long)__double_as_longlong(local_err));
@@ -245,14 +223,24 @@ __global__ void rkf45_set_dt_kernel(RKFControl* c, double dt, int reset)
         c->trials = 0ull;
         c->accepted_steps = 0ull;
         c->failed_steps = 0ull;
+        c->attempts = 0u;
+        c->accepted = 0;
+        c->err_bits = 0ull;
     }
 }
 
-__global__ void rkf45_begin_kernel(RKFControl* c)
+// r^(1/5) for r in [1e-4, 100]: the FP32 power refined by two Newton steps on
+// x^5 = r in FP64 (relative error 1e-7 -> 2e-14 -> below one ulp).  The FP64
+// pow() alone took most of the controller's 5.3 us on one thread.
+__device__ __forceinline__ double fifth_root(double r)
 {
-    c->attempts = 0u;
-    c->accepted = 0;
-    c->err_bits = 0ull;
+    double x = (double)powf((float)r, 0.2f);
+#pragma unroll
+    for (int i = 0; i < 2; i++) {
+        const double x2 = x * x, x4 = x2 * x2;
+        x += (r - x4 * x) / (5.0 * x4);
+    }
+    return x;
 }
 
 __global__ void rkf45_control_kernel(RKFControl* c, double tol, double dt_min, double dt_max, int* status,
@@ -260,27 +248,33 @@ __global__ void rkf45_control_kernel(RKFControl* c, double tol, double dt_min, d
 {
     const double err = __longlong_as_double((long long)c->err_bits);
     const double h = c->dt;
-    const double fac = err == 0.0 ? 2.0 : fmin(2.0, fmax(0.2, 0.9 * pow(tol / err, 0.2)));
+    // clip(0.9 (tol/err)^(1/5), 0.2, 2): the root only where neither bound holds anyway
+    // (0.9^5 55 > 2^5, 0.9^5 5e-4 < 0.2^5; a NaN shrinks the step)
+    const double ratio = tol / err;
+    double fac = 0.2;
+    if (err == 0.0 || ratio >= 55.0) fac = 2.0;
+    else if (ratio > 5e-4) fac = fmin(2.0, fmax(0.2, 0.9 * fifth_root(ratio)));
     const double hn = fmin(dt_max, fmax(dt_min, h * fac));
     const bool acc = err <= tol || h <= dt_min;
     const unsigned int tries = c->attempts + 1u;
-    c->attempts = tries;
+    const bool again = !acc && tries < RKF_MAX_TRIALS;
+    c->attempts = again ? tries : 0u;  // the next step starts with none
+    c->accepted = acc ? 1 : 0;
     c->err = err;
     c->trials += 1ull;
     c->err_bits = 0ull;
     c->dt = hn;
     if (acc) {
-        c->accepted = 1;
         c->dt_used = h;
         c->t += h;
         c->accepted_steps += 1ull;
-    } else if (tries >= RKF_MAX_TRIALS) {
+    } else if (!again) {
         c->failed_steps += 1ull;
         if (status) atomicCAS(status, 0, -6);  // BORIS_ERR_STEP_CONTROL
     }
     // repeat the trial only while it is rejected and trials remain: the loop
     // ends after at most RKF_MAX_TRIALS passes whatever the error is
-    cudaGraphSetConditional(loop, (!acc && tries < RKF_MAX_TRIALS) ? 1u : 0u);
+    cudaGraphSetConditional(loop, again ? 1u : 0u);
 }
 
 template <typename T>
@@ -306,7 +300,7 @@ __global__ void __launch_bounds__(256) energy_kernel(LLGArgs<T> a, const T* __re
         const double mc[3] = {(double)m[i], (double)m[n + i], (double)m[2 * n + i]};
         double lap[3], w[3];
         // neighbours (or boundary ghosts) in FP64; without DMI the ghost is the cell itself
-        ext_exchange_dmi<double>(a, m, i, x, y, z, mc, lap, w);
+        ext_exchange_dmi<double>(a, m, (unsigned)i, x, y, z, mc, lap, w);
         const double Ms = a.ms_map ? (double)a.ms_map[i] : (double)a.Ms;
         const double Ku = a.ku_map ? (double)a.ku_map[i] : (double)a.Ku;
         const double me = mc[0] * a.e[0] + mc[1] * a.e[1] + mc[2] * a.e[2];
@@ -381,7 +375,7 @@ __device__ __forceinline__ void ml_field_and_rhs(const LLGArgs<T>& a, const MLTa
 #pragma unroll
     for (int c = 0; c < 3; c++) H[c] = Hd[vi[c]] + cex * lap[c] + can * a.e[c] + a.Hext[c];
     if (a.extra) {
-        ext_local_field<T>(a, m, Ms, H);
+        ext_local_field<T>(a, m, inv, H);
         // surface exchange (Eq. 5): the top plane of layer l with the bottom
         // plane of layer l + 1 where they overlap in-plane, and the reverse;
         // Delta = this cell's z size
@@ -505,13 +499,27 @@ cudaError_t launch_rk4_stage(const LLGArgs<T>& a, int s, const T* ms, const T* H
                              cudaStream_t st)
 {
     if constexpr (sizeof(T) == 4) {
-        if (a.nx % 4 == 0 && !a.extra) {
+        // quads from 400 k cells on: below, four times the threads with a quarter of
+        // the work each are the shorter chain (256 x 64 x 1 3.2 against 2.6 us, 256 x 256
+        // x 4 4.3 against 3.8; 512 x 512 x 4 11.7 against 15)
+        if (a.nx % 4 == 0 && !a.extra && a.ncell >= 400000) {
             if (a.pbc) rk4_stage_quad_kernel<true><<<grid_for(a.ncell / 4), 256, 0, st>>>(a, s, ms, Hd, m0, acc, mnext);
             else rk4_stage_quad_kernel<false><<<grid_for(a.ncell / 4), 256, 0, st>>>(a, s, ms, Hd, m0, acc, mnext);
             return cudaGetLastError();
         }
     }
-    rk4_stage_kernel<T><<<grid_for(a.ncell), 256, 0, st>>>(a, s, ms, Hd, m0, acc, mnext);
+    const int g = grid_for(a.ncell);
+    switch (a.extra ? s + 4 : s) {
+#define RK4_STAGE(S)                                                                                 \
+    case S: rk4_stage_kernel<T, false, S><<<g, 256, 0, st>>>(a, ms, Hd, m0, acc, mnext); break;      \
+    case S + 4: rk4_stage_kernel<T, true, S><<<g, 256, 0, st>>>(a, ms, Hd, m0, acc, mnext); break;
+        RK4_STAGE(0)
+        RK4_STAGE(1)
+        RK4_STAGE(2)
+        RK4_STAGE(3)
+#undef RK4_STAGE
+    default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 
@@ -519,19 +527,26 @@ template <typename T>
 cudaError_t launch_rkf45_stage(const LLGArgs<T>& a, int s, const T* ms, const T* Hd, const T* m0, T* kbuf, T* mnext,
                                unsigned long long* err_bits, cudaStream_t st)
 {
-    rkf45_stage_kernel<T><<<grid_for(a.ncell), 256, 0, st>>>(a, s, ms, Hd, m0, kbuf, mnext, err_bits);
+    const int g = grid_for(a.ncell);
+    switch (a.extra ? s + 6 : s) {
+#define RKF_STAGE(S)                                                                                                 \
+    case S: rkf45_stage_kernel<T, false, S><<<g, 256, 0, st>>>(a, ms, Hd, m0, kbuf, mnext, err_bits); break;         \
+    case S + 6: rkf45_stage_kernel<T, true, S><<<g, 256, 0, st>>>(a, ms, Hd, m0, kbuf, mnext, err_bits); break;
+        RKF_STAGE(0)
+        RKF_STAGE(1)
+        RKF_STAGE(2)
+        RKF_STAGE(3)
+        RKF_STAGE(4)
+        RKF_STAGE(5)
+#undef RKF_STAGE
+    default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 
 cudaError_t launch_rkf45_set_dt(RKFControl* c, double dt, bool reset_counters, cudaStream_t st)
 {
     rkf45_set_dt_kernel<<<1, 1, 0, st>>>(c, dt, reset_counters ? 1 : 0);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_rkf45_begin(RKFControl* c, cudaStream_t st)
-{
-    rkf45_begin_kernel<<<1, 1, 0, st>>>(c);
     return cudaGetLastError();
 }
 

@@ -13,7 +13,7 @@ template <typename T>
 __device__ __forceinline__ void rhs_local(const LLGArgs<T>& a, const T m[3], const T lap[3], const T hd[3], T Ms, T Ku,
                                           T k[3])
 {
-    const T inv = T(1) / (T(MU0_D) * Ms);
+    const T inv = a.ms_map ? T(1) / (T(MU0_D) * Ms) : a.inv_ms;
     const T cex = T(2) * a.A * inv;
     const T me = m[0] * a.e[0] + m[1] * a.e[1] + m[2] * a.e[2];
     const T can = T(2) * Ku * inv * me;
@@ -35,17 +35,10 @@ __device__ __forceinline__ void rhs_local(const LLGArgs<T>& a, const T m[3], con
 // differences both use it (without DMI the ghost is m: homogeneous Neumann).
 // TC is the arithmetic type (T for the stage kernels, double for energies).
 // ---------------------------------------------------------------------------
+// The value beyond an open face along `axis` on side sgn: m, or with DMI its ghost.
 template <typename TC, typename T>
-__device__ __forceinline__ void nb_or_ghost(const LLGArgs<T>& a, const T* __restrict__ ms, bool inside, size_t j,
-                                            int axis, int sgn, const TC m[3], TC out[3])
+__device__ __forceinline__ void face_ghost(const LLGArgs<T>& a, int axis, int sgn, const TC m[3], TC out[3])
 {
-    const size_t n = a.ncell;
-    if (inside) {
-        out[0] = (TC)ms[j];
-        out[1] = (TC)ms[n + j];
-        out[2] = (TC)ms[2 * n + j];
-        return;
-    }
     out[0] = m[0];
     out[1] = m[1];
     out[2] = m[2];
@@ -74,23 +67,67 @@ __device__ __forceinline__ void nb_or_ghost(const LLGArgs<T>& a, const T* __rest
     }
 }
 
+// The six neighbours of a cell: index, and whether there is one (a periodic
+// axis wraps to the opposite face; a missing neighbour has the cell's own
+// index).  Loading all six unconditionally keeps them in flight together: with
+// a branch around each load they came one after the other, six trips to L2
+// (256 x 64 x 1 RKF45 stage 5.3 us, 512 x 512 x 1 DMI stage 9.2 us).
+struct Neighbours {
+    unsigned xm, xp, ym, yp, zm, zp;
+    bool hxm, hxp, hym, hyp, hzm, hzp;
+};
+template <typename T>
+__device__ __forceinline__ Neighbours neighbours(const LLGArgs<T>& a, unsigned i, int x, int y, int z)
+{
+    const unsigned sy = a.nx, sz = (unsigned)a.nx * a.ny;
+    const bool px = a.pbc & 1, py = a.pbc & 2, pz = a.pbc & 4;
+    Neighbours q;
+    q.hxm = x > 0 || px;
+    q.hxp = x < a.nx - 1 || px;
+    q.hym = y > 0 || py;
+    q.hyp = y < a.ny - 1 || py;
+    q.hzm = z > 0 || pz;
+    q.hzp = z < a.nz - 1 || pz;
+    q.xm = x > 0 ? i - 1 : px ? i + (a.nx - 1) : i;
+    q.xp = x < a.nx - 1 ? i + 1 : px ? i - (a.nx - 1) : i;
+    q.ym = y > 0 ? i - sy : py ? i + (a.ny - 1) * sy : i;
+    q.yp = y < a.ny - 1 ? i + sy : py ? i - (a.ny - 1) * sy : i;
+    q.zm = z > 0 ? i - sz : pz ? i + (a.nz - 1) * sz : i;
+    q.zp = z < a.nz - 1 ? i + sz : pz ? i - (a.nz - 1) * sz : i;
+    return q;
+}
+
 // Exchange Laplacian sum_axes (m_+ + m_- - 2m)/h^2 and the DMI vector w with
 // H_dmi = (2D/(mu0 Ms)) w: bulk w = -curl m, interfacial w = (-dmz/dx,
 // -dmz/dy, dmx/dx + dmy/dy), derivatives (m_+ - m_-)/(2h).
 template <typename TC, typename T>
-__device__ __forceinline__ void ext_exchange_dmi(const LLGArgs<T>& a, const T* __restrict__ ms, size_t i, int x, int y,
+__device__ __forceinline__ void ext_exchange_dmi(const LLGArgs<T>& a, const T* __restrict__ ms, unsigned i, int x, int y,
                                                  int z, const TC m[3], TC lap[3], TC w[3])
 {
-    const size_t sy = a.nx, sz = (size_t)a.nx * a.ny;
-    const bool px = a.pbc & 1, py = a.pbc & 2, pz = a.pbc & 4;
+    const unsigned n = (unsigned)a.ncell;
+    const Neighbours q = neighbours(a, i, x, y, z);
     TC xm[3], xp[3], ym[3], yp[3], zm[3], zp[3];
-    // a periodic axis wraps to the cell on the opposite face
-    nb_or_ghost<TC>(a, ms, x > 0 || px, x > 0 ? i - 1 : i + (a.nx - 1), 0, -1, m, xm);
-    nb_or_ghost<TC>(a, ms, x < a.nx - 1 || px, x < a.nx - 1 ? i + 1 : i - (a.nx - 1), 0, 1, m, xp);
-    nb_or_ghost<TC>(a, ms, y > 0 || py, y > 0 ? i - sy : i + (a.ny - 1) * sy, 1, -1, m, ym);
-    nb_or_ghost<TC>(a, ms, y < a.ny - 1 || py, y < a.ny - 1 ? i + sy : i - (a.ny - 1) * sy, 1, 1, m, yp);
-    nb_or_ghost<TC>(a, ms, z > 0 || pz, z > 0 ? i - sz : i + (a.nz - 1) * sz, 2, -1, m, zm);
-    nb_or_ghost<TC>(a, ms, z < a.nz - 1 || pz, z < a.nz - 1 ? i + sz : i - (a.nz - 1) * sz, 2, 1, m, zp);
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        xm[c] = (TC)ms[c * n + q.xm];
+        xp[c] = (TC)ms[c * n + q.xp];
+        ym[c] = (TC)ms[c * n + q.ym];
+        yp[c] = (TC)ms[c * n + q.yp];
+        zm[c] = (TC)ms[c * n + q.zm];
+        zp[c] = (TC)ms[c * n + q.zp];
+    }
+    // ghosts only where a face is open (along z they differ from m with bulk DMI only)
+    if (a.dmi && (!(q.hxm && q.hxp && q.hym && q.hyp) || (a.dmi == 1 && !(q.hzm && q.hzp)))) {
+        auto open = [&](bool has, int axis, int sgn, TC (&v)[3]) {
+            if (!has) face_ghost<TC>(a, axis, sgn, m, v);
+        };
+        open(q.hxm, 0, -1, xm);
+        open(q.hxp, 0, 1, xp);
+        open(q.hym, 1, -1, ym);
+        open(q.hyp, 1, 1, yp);
+        open(q.hzm, 2, -1, zm);
+        open(q.hzp, 2, 1, zp);
+    }
 #pragma unroll
     for (int c = 0; c < 3; c++)
         lap[c] = (xp[c] + xm[c] - TC(2) * m[c]) * (TC)a.ihx2 + (yp[c] + ym[c] - TC(2) * m[c]) * (TC)a.ihy2 +
@@ -98,7 +135,16 @@ __device__ __forceinline__ void ext_exchange_dmi(const LLGArgs<T>& a, const T* _
     w[0] = w[1] = w[2] = TC(0);
     if (a.dmi == 0) return;
     TC dx[3], dy[3], dz[3];
-    const TC ix = TC(0.5) / (TC)a.hx, iy = TC(0.5) / (TC)a.hy, iz = TC(0.5) / (TC)a.hz;
+    TC ix, iy, iz;  // 1/(2h)
+    if constexpr (sizeof(TC) == sizeof(T)) {
+        ix = a.i2hx;
+        iy = a.i2hy;
+        iz = a.i2hz;
+    } else {
+        ix = TC(0.5) / (TC)a.hx;
+        iy = TC(0.5) / (TC)a.hy;
+        iz = TC(0.5) / (TC)a.hz;
+    }
 #pragma unroll
     for (int c = 0; c < 3; c++) {
         dx[c] = (xp[c] - xm[c]) * ix;
@@ -117,11 +163,11 @@ __device__ __forceinline__ void ext_exchange_dmi(const LLGArgs<T>& a, const T* _
 }
 
 // Local further terms added to H: (4 K2/(mu0 Ms)) (1 - (m.e)^2)(m.e) e and the
-// cubic field -(2 Kc1/(mu0 Ms)) [e1 a(b^2 + c^2) + ...] - (2 Kc2/(mu0 Ms)) [e1 a b^2 c^2 + ...].
+// cubic field -(2 Kc1/(mu0 Ms)) [e1 a(b^2 + c^2) + ...] - (2 Kc2/(mu0 Ms)) [e1 a b^2 c^2 + ...];
+// inv = 1/(mu0 Ms).
 template <typename TC, typename T>
-__device__ __forceinline__ void ext_local_field(const LLGArgs<T>& a, const TC m[3], TC Ms, TC H[3])
+__device__ __forceinline__ void ext_local_field(const LLGArgs<T>& a, const TC m[3], TC inv, TC H[3])
 {
-    const TC inv = TC(1) / (TC(MU0_D) * Ms);
     if (a.K2 != T(0)) {
         const TC me = m[0] * (TC)a.e[0] + m[1] * (TC)a.e[1] + m[2] * (TC)a.e[2];
         const TC f = TC(4) * (TC)a.K2 * inv * (TC(1) - me * me) * me;
@@ -179,7 +225,7 @@ __device__ __forceinline__ void philox4x32_10(unsigned int c[4], unsigned int k0
 
 // three standard normals of cell i at the plan's current step
 template <typename T>
-__device__ __forceinline__ void thermal_normals(const LLGArgs<T>& a, size_t i, T g[3])
+__device__ __forceinline__ void thermal_normals(const LLGArgs<T>& a, unsigned i, T g[3])
 {
     const unsigned long long s = *a.step;
     unsigned int c[4] = {(unsigned int)i, (unsigned int)s, (unsigned int)(s >> 32), 0u};
@@ -212,84 +258,97 @@ __device__ __forceinline__ void rhs_from_field(const LLGArgs<T>& a, const T m[3]
     for (int c = 0; c < 3; c++) k[c] = -a.gp * (mxH[c] + a.alpha * mmH[c]);
 }
 
-// m = ms[i]; k = -g' [m x H + alpha m x (m x H)], H = hd + exchange + anisotropy + Hext
-// (+ the further terms when a.extra is set).
+// 1 / (mu0 Ms) of a cell: the host's value where Ms is uniform
 template <typename T>
-__device__ __forceinline__ void cell_rhs(const LLGArgs<T>& a, const T* __restrict__ ms, const T hd[3], size_t i, int x,
+__device__ __forceinline__ T inv_mu0_ms(const LLGArgs<T>& a, T Ms)
+{
+    return a.ms_map ? T(1) / (T(MU0_D) * Ms) : a.inv_ms;
+}
+
+// m = ms[i]; k = -g' [m x H + alpha m x (m x H)], H = hd + exchange + anisotropy + Hext
+// (EXTRA: + the further terms).
+template <bool EXTRA, typename T>
+__device__ __forceinline__ void cell_rhs(const LLGArgs<T>& a, const T* __restrict__ ms, const T hd[3], unsigned i, int x,
                                          int y, int z, T m[3], T k[3])
 {
-    const size_t n = a.ncell;
+    const unsigned n = (unsigned)a.ncell;
     m[0] = ms[i];
     m[1] = ms[n + i];
     m[2] = ms[2 * n + i];
-    if (a.extra) {
-        T lap[3], w[3];
+    const T Ms = a.ms_map ? a.ms_map[i] : a.Ms;
+    const T Ku = a.ku_map ? a.ku_map[i] : a.Ku;
+    if constexpr (EXTRA) {
+        T lap[3], w[3], ha[3] = {T(0), T(0), T(0)};
+        if (a.hadd) {
+#pragma unroll
+            for (int c = 0; c < 3; c++) ha[c] = a.hadd[c * n + i];
+        }
         ext_exchange_dmi<T>(a, ms, i, x, y, z, m, lap, w);
-        const T Ms = a.ms_map ? a.ms_map[i] : a.Ms;
-        const T Ku = a.ku_map ? a.ku_map[i] : a.Ku;
-        const T inv = T(1) / (T(MU0_D) * Ms);
+        const T inv = inv_mu0_ms(a, Ms);
         const T cex = T(2) * a.A * inv, cd = T(2) * a.D * inv;
         const T me = m[0] * a.e[0] + m[1] * a.e[1] + m[2] * a.e[2];
         const T can = T(2) * Ku * inv * me;
         T H[3];
 #pragma unroll
         for (int c = 0; c < 3; c++) H[c] = hd[c] + cex * lap[c] + cd * w[c] + can * a.e[c] + a.Hext[c];
-        ext_local_field<T>(a, m, Ms, H);
+        ext_local_field<T>(a, m, inv, H);
         if (a.hadd) {
 #pragma unroll
-            for (int c = 0; c < 3; c++) H[c] += a.hadd[c * n + i];
+            for (int c = 0; c < 3; c++) H[c] += ha[c];
         }
         if (a.th_s0 > T(0)) {
             T g[3];
             thermal_normals(a, i, g);
-            const T sg = a.th_s0 / sqrt(Ms);
+            const T sg = a.ms_map ? a.th_s0 / sqrt(Ms) : a.th_sg;
 #pragma unroll
             for (int c = 0; c < 3; c++) H[c] += sg * g[c];
         }
         rhs_from_field(a, m, H, k);
         return;
     }
-    T lap[3] = {T(0), T(0), T(0)};
-    auto nb = [&](size_t j, T w) {
-        lap[0] += w * (ms[j] - m[0]);
-        lap[1] += w * (ms[n + j] - m[1]);
-        lap[2] += w * (ms[2 * n + j] - m[2]);
-    };
-    const size_t sy = a.nx, sz = (size_t)a.nx * a.ny;
-    // a missing neighbour is the cell itself (homogeneous Neumann), or the
-    // cell on the opposite face along a periodic axis
-    if (x > 0) nb(i - 1, a.ihx2);
-    else if (a.pbc & 1) nb(i + (a.nx - 1), a.ihx2);
-    if (x < a.nx - 1) nb(i + 1, a.ihx2);
-    else if (a.pbc & 1) nb(i - (a.nx - 1), a.ihx2);
-    if (y > 0) nb(i - sy, a.ihy2);
-    else if (a.pbc & 2) nb(i + (a.ny - 1) * sy, a.ihy2);
-    if (y < a.ny - 1) nb(i + sy, a.ihy2);
-    else if (a.pbc & 2) nb(i - (a.ny - 1) * sy, a.ihy2);
-    if (z > 0) nb(i - sz, a.ihz2);
-    else if (a.pbc & 4) nb(i + (a.nz - 1) * sz, a.ihz2);
-    if (z < a.nz - 1) nb(i + sz, a.ihz2);
-    else if (a.pbc & 4) nb(i - (a.nz - 1) * sz, a.ihz2);
-    const T Ms = a.ms_map ? a.ms_map[i] : a.Ms;
-    const T Ku = a.ku_map ? a.ku_map[i] : a.Ku;
+    // a missing neighbour is the cell itself (homogeneous Neumann): its term is zero
+    const Neighbours q = neighbours(a, i, x, y, z);
+    T nb[3][6], lap[3];
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const T* f = ms + c * n;
+        nb[c][0] = f[q.xm];
+        nb[c][1] = f[q.xp];
+        nb[c][2] = f[q.ym];
+        nb[c][3] = f[q.yp];
+        nb[c][4] = f[q.zm];
+        nb[c][5] = f[q.zp];
+    }
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        T l = a.ihx2 * (nb[c][0] - m[c]);
+        l += a.ihx2 * (nb[c][1] - m[c]);
+        l += a.ihy2 * (nb[c][2] - m[c]);
+        l += a.ihy2 * (nb[c][3] - m[c]);
+        l += a.ihz2 * (nb[c][4] - m[c]);
+        l += a.ihz2 * (nb[c][5] - m[c]);
+        lap[c] = l;
+    }
     rhs_local(a, m, lap, hd, Ms, Ku, k);
 }
 
-template <typename T>
+template <bool EXTRA, typename T>
 __device__ __forceinline__ void field_and_rhs(const LLGArgs<T>& a, const T* __restrict__ ms, const T* __restrict__ Hd,
-                                              size_t i, int x, int y, int z, T m[3], T k[3])
+                                              unsigned i, int x, int y, int z, T m[3], T k[3])
 {
-    const size_t n = a.ncell;
+    const unsigned n = (unsigned)a.ncell;
     const T hd[3] = {Hd[i], Hd[n + i], Hd[2 * n + i]};
-    cell_rhs(a, ms, hd, i, x, y, z, m, k);
+    cell_rhs<EXTRA>(a, ms, hd, i, x, y, z, m, k);
 }
 
-// RK4 stage combine for cell i (stage s in 0..3; m = stage state, k = its rate).
+// RK4 stage combine for cell i (stage s in 0..3; m = stage state, k = its
+// rate), from b = m0 and ac = acc of the cell (read from s = 1 on).
 template <typename T>
-__device__ __forceinline__ void rk4_combine(const LLGArgs<T>& a, int s, size_t i, const T m[3], const T k[3],
-                                            T* __restrict__ m0, T* __restrict__ acc, T* __restrict__ mnext)
+__device__ __forceinline__ void rk4_combine(const LLGArgs<T>& a, int s, unsigned i, const T m[3], const T k[3],
+                                            const T b[3], const T ac[3], T* __restrict__ m0, T* __restrict__ acc,
+                                            T* __restrict__ mnext)
 {
-    const size_t n = a.ncell;
+    const unsigned n = (unsigned)a.ncell;
     if (s == 0) {
 #pragma unroll
         for (int c = 0; c < 3; c++) {
@@ -300,16 +359,85 @@ __device__ __forceinline__ void rk4_combine(const LLGArgs<T>& a, int s, size_t i
         const T cdt = s == 1 ? T(0.5) * a.dt : a.dt;
 #pragma unroll
         for (int c = 0; c < 3; c++) {
-            acc[c * n + i] += T(2) * k[c];
-            mnext[c * n + i] = m0[c * n + i] + cdt * k[c];
+            acc[c * n + i] = ac[c] + T(2) * k[c];
+            mnext[c * n + i] = b[c] + cdt * k[c];
         }
     } else {
         T v[3];
 #pragma unroll
-        for (int c = 0; c < 3; c++) v[c] = m0[c * n + i] + a.dt * (T(1) / T(6)) * (acc[c * n + i] + k[c]);
+        for (int c = 0; c < 3; c++) v[c] = b[c] + a.dt * (T(1) / T(6)) * (ac[c] + k[c]);
         const T inv = T(1) / sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
 #pragma unroll
         for (int c = 0; c < 3; c++) m0[c * n + i] = v[c] * inv;
+    }
+}
+
+// Runge-Kutta-Fehlberg 4(5) (Fehlberg's published tableau): stage s state =
+// m0 + dt sum_j A[s][j] k_j; 4th/5th order weights B4, B5.
+__host__ __device__ constexpr double rkf_a(int s, int j)
+{
+    constexpr double A[6][5] = {
+        {0, 0, 0, 0, 0},
+        {1.0 / 4, 0, 0, 0, 0},
+        {3.0 / 32, 9.0 / 32, 0, 0, 0},
+        {1932.0 / 2197, -7200.0 / 2197, 7296.0 / 2197, 0, 0},
+        {439.0 / 216, -8.0, 3680.0 / 513, -845.0 / 4104, 0},
+        {-8.0 / 27, 2.0, -3544.0 / 2565, 1859.0 / 4104, -11.0 / 40},
+    };
+    return A[s][j];
+}
+__host__ __device__ constexpr double rkf_b4(int j)
+{
+    constexpr double B[6] = {25.0 / 216, 0.0, 1408.0 / 2565, 2197.0 / 4104, -1.0 / 5, 0.0};
+    return B[j];
+}
+__host__ __device__ constexpr double rkf_b5(int j)
+{
+    constexpr double B[6] = {16.0 / 135, 0.0, 6656.0 / 12825, 28561.0 / 56430, -9.0 / 50, 2.0 / 55};
+    return B[j];
+}
+
+// Stage S of cell i with rate k, from b = m0 and the earlier rates kj[c][j]:
+// stores k_S and the next stage state m0 + dt sum_{j <= S} a_{S+1,j} k_j in mnext;
+// S = 5: the normalised 4th-order solution, and err raised to |m5 - m4| =
+// dt |sum_j (b5_j - b4_j) k_j| (FP64).
+template <int S, typename T>
+__device__ __forceinline__ void rkf45_update(unsigned n, unsigned i, const T k[3], T dt, const T b[3],
+                                             const T (&kj)[3][S > 0 ? S : 1], T* __restrict__ kbuf,
+                                             T* __restrict__ mnext, double& err)
+{
+    if constexpr (S < 5) {
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            kbuf[(size_t)(S * 3 + c) * n + i] = k[c];
+            T v = b[c];
+#pragma unroll
+            for (int j = 0; j < S; j++) v += dt * T(rkf_a(S + 1, j)) * kj[c][j];
+            v += dt * T(rkf_a(S + 1, S)) * k[c];
+            mnext[c * n + i] = v;
+        }
+    } else {
+        T v[3];
+        double e2 = 0.0;
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            kbuf[(size_t)(S * 3 + c) * n + i] = k[c];
+            T s4 = T(0);
+            double d = 0.0;
+#pragma unroll
+            for (int j = 0; j < 6; j++) {
+                const T q = j == 5 ? k[c] : kj[c][j < S ? j : 0];
+                s4 += T(rkf_b4(j)) * q;
+                d += (rkf_b5(j) - rkf_b4(j)) * (double)q;
+            }
+            v[c] = b[c] + dt * s4;
+            d *= (double)dt;
+            e2 += d * d;
+        }
+        err = fmax(err, sqrt(e2));
+        const T inv = T(1) / sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+#pragma unroll
+        for (int c = 0; c < 3; c++) mnext[c * n + i] = v[c] * inv;
     }
 }
 

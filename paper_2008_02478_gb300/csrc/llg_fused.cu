@@ -91,8 +91,17 @@ __global__ void __launch_bounds__(FT, 2)
         const size_t i = ((size_t)z * ny + y) * nx + x;
         const float hd[3] = {Hs[t * HROW + x], Hs[(FY + t) * HROW + x], Hs[(2 * FY + t) * HROW + x]};
         float m[3], k[3];
-        cell_rhs(a, ms, hd, i, x, y, z, m, k);
-        rk4_combine(a, s, i, m, k, m0, acc, mnext);
+        cell_rhs<false>(a, ms, hd, i, x, y, z, m, k);
+        const size_t n = a.ncell;
+        float b[3] = {}, ac[3] = {};
+        if (s > 0) {
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                b[c] = m0[c * n + i];
+                ac[c] = acc[c * n + i];
+            }
+        }
+        rk4_combine(a, s, i, m, k, b, ac, m0, acc, mnext);
     }
 }
 

@@ -14,6 +14,7 @@ struct LLGArgs {
     size_t ncell;
     T ihx2, ihy2, ihz2;  // 1/h^2 per axis
     T Ms, Ku, A;         // uniform values (used when the map is NULL)
+    T inv_ms;            // 1 / (mu0 Ms) of the uniform Ms
     const T* ms_map;
     const T* ku_map;
     T e[3];
@@ -31,10 +32,12 @@ struct LLGArgs {
     T D;                // DMI constant
     T kD;               // D / (2A): boundary slope of the non-homogeneous Neumann condition
     T hx, hy, hz;       // cell sizes (central differences, boundary ghosts)
+    T i2hx, i2hy, i2hz; // 1/(2h)
     T J1, J2;           // surface exchange between consecutive multi-mesh layers (Eq. 5)
     int pbc;            // periodic axes (bit 0 x, 1 y, 2 z): stencil neighbours wrap around
     // thermal field: sigma_i = th_s0 / sqrt(Ms_i) (0: off); Philox key and step counter
     T th_s0;
+    T th_sg;            // th_s0 / sqrt(Ms) of the uniform Ms
     unsigned int seed_lo, seed_hi;
     const unsigned long long* step;
     const T* hadd;      // additive field map [3][nz][ny][nx] (e.g. an Oersted field) or NULL
@@ -63,10 +66,9 @@ struct RKFControl {
     unsigned long long failed_steps;  // steps that ran out of trials
 };
 constexpr unsigned int RKF_MAX_TRIALS = 16;
-// the next step to try
+// the next step to try; reset: also clears the counters, the error maximum and the
+// trial count (the controller leaves both cleared after every step)
 cudaError_t launch_rkf45_set_dt(RKFControl* c, double dt, bool reset_counters, cudaStream_t st);
-// start of a step: no trial yet, error max cleared
-cudaError_t launch_rkf45_begin(RKFControl* c, cudaStream_t st);
 // after a trial; sets the trial loop's condition (1: repeat) and latches
 // BORIS_ERR_STEP_CONTROL in *status when RKF_MAX_TRIALS trials were rejected
 cudaError_t launch_rkf45_control(RKFControl* c, double tol, double dt_min, double dt_max, int* status,

@@ -166,7 +166,7 @@ cudaError_t x_set_attr(const MixedPlan& m)
             e = cudaFuncSetAttribute(x_inv_kernel<T, Len<r1, r2, r3, __VA_ARGS__>>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
                                      227 * 1024);                                                                     \
         break;
-        BORIS_LENGTHS(X)
+        BORIS_LENGTHS_FINE(X)
 #undef X
     }
     return e;
@@ -183,7 +183,7 @@ cudaError_t launch_mixed_x_fwd(const MixedPlan& m, const T* M, const T* ms_map, 
     switch (m.x.id) {
 #define X(i, r1, r2, r3, ...) \
     case i: x_fwd_kernel<T, Len<r1, r2, r3, __VA_ARGS__>><<<l.grid, l.threads, l.smem, st>>>(l.a); break;
-        BORIS_LENGTHS(X)
+        BORIS_LENGTHS_FINE(X)
 #undef X
     }
     return cudaGetLastError();
@@ -197,7 +197,7 @@ cudaError_t launch_mixed_x_inv(const MixedPlan& m, const typename Cx<T>::t* X_, 
     switch (m.x.id) {
 #define X(i, r1, r2, r3, ...) \
     case i: x_inv_kernel<T, Len<r1, r2, r3, __VA_ARGS__>><<<l.grid, l.threads, l.smem, st>>>(l.a); break;
-        BORIS_LENGTHS(X)
+        BORIS_LENGTHS_FINE(X)
 #undef X
     }
     return cudaGetLastError();
