@@ -262,7 +262,7 @@ int boris_llg_step_f64(boris_plan p, double* m, const boris_llg_params* prm, dou
  *   Landau-Lifshitz right-hand side, exchange (the Neumann Laplacian is
  *   symmetric), anisotropy and the demagnetising operator, which is
  *   self-adjoint so each transpose is one more demag application.
- *   prm->method must be BORIS_RK4.  Workspace: 18 fields, allocated once.
+ *   prm->method must be BORIS_RK4.  Workspace: 14 fields and a map, allocated once.
  */
 int boris_llg_step_backward(boris_plan p, const float* m_in, const boris_llg_params* prm, double dt,
                             const float* g_m_out, float* g_m_in, float* g_Ms, float* g_Ku);

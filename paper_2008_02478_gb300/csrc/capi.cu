@@ -127,8 +127,8 @@ struct boris_plan_s {
     float* Mf = nullptr;    // frame fields [3][Z][NY][NX]
     float* Hf = nullptr;
     int ml_unique = 0;
-    // adjoint workspace: stage states m2..m4, stage fields, stage derivatives,
-    // stage cotangents, and three scratch fields
+    // adjoint workspace: stage states m2..m4, fields and derivatives of stages 1..3, gv,
+    // four scratch fields and 1/(mu0 Ms)
     void* bw = nullptr;
     size_t bytes = 0;
     // optional per-kernel CUDA-event timing (boris_profile_enable)
@@ -680,34 +680,39 @@ int llg_backward_t(boris_plan p, const T* m_in, const boris_llg_params* prm, dou
     LLGArgs<T> a;
     if ((rc = check_params<T>(p, prm, &a, dt))) return rc;
     const size_t n3 = 3 * ncell(p);
-    if (!p->bw && (rc = dev_alloc(p, &p->bw, 18 * n3 * sizeof(T)))) return rc;
+    if (!p->bw && (rc = dev_alloc(p, &p->bw, (14 * n3 + (n3 / 3 + 3) / 4 * 4) * sizeof(T)))) return rc;
     T* w = (T*)p->bw;
     T* mst[4] = {(T*)m_in, w, w + n3, w + 2 * n3};
-    T* Hs = w + 3 * n3;   // 4 x n3
-    T* ks = w + 7 * n3;   // 4 x n3
-    T* gk = w + 11 * n3;  // 4 x n3
-    T* gH = w + 15 * n3;
-    T* DgH = w + 16 * n3;
-    T* gml = w + 17 * n3;
+    T* Hs = w + 3 * n3;  // 3 x n3
+    T* ks = w + 6 * n3;  // 3 x n3
+    T* gvb = w + 9 * n3;
+    T* gH[2] = {w + 10 * n3, w + 11 * n3};  // alternate between stages
+    T* DgH = w + 12 * n3;
+    T* gml = w + 13 * n3;
+    T* imap = w + 14 * n3;
     T* Hd = (T*)p->Hd;
     const T* ms_map = (const T*)prm->Ms_map;
-    for (int s = 0; s < 4; s++) {
+    if (ms_map) CUDA_TRY(timed(p, 3, [&] { return launch_bwd_inv_ms<T>(a, imap, p->stream); }));
+    for (int s = 0; s < 3; s++) {
         if ((rc = demag_apply_t<T>(p, mst[s], ms_map, a.Ms, Hd))) return rc;
         CUDA_TRY(timed(p, 3, [&] {
-            return launch_fwd_stage<T>(a, s, mst[s], Hd, m_in, Hs + s * n3, ks + s * n3, s < 3 ? mst[s + 1] : nullptr,
-                                       p->stream);
+            return launch_fwd_stage<T>(a, s, mst[s], Hd, m_in, Hs + s * n3, ks + s * n3, mst[s + 1], p->stream);
         }));
     }
+    if ((rc = demag_apply_t<T>(p, mst[3], ms_map, a.Ms, Hd))) return rc;
     CUDA_TRY(timed(p, 3, [&] {
-        return launch_bwd_start<T>(a, m_in, ks, ks + n3, ks + 2 * n3, ks + 3 * n3, g_out, g_in, gk, p->stream);
+        return launch_bwd_turn<T>(a, mst[3], Hd, m_in, ks, g_out, g_in, gvb, gH[1], gml, p->stream);
     }));
+    // gk_{s-1} = wk[s-1] gv + back[s] gm_s
     const T back[4] = {T(0), T(0.5 * dt), T(0.5 * dt), T(dt)};
+    const T wk[4] = {a.dt / T(6), a.dt / T(3), a.dt / T(3), a.dt / T(6)};
     for (int s = 3; s >= 0; s--) {
-        CUDA_TRY(timed(p, 3, [&] { return launch_bwd_local<T>(a, mst[s], Hs + s * n3, gk + s * n3, gH, gml, p->stream); }));
-        if ((rc = demag_apply_t<T>(p, gH, nullptr, T(1), DgH))) return rc;
+        T* g = gH[s & 1];
+        if ((rc = demag_apply_t<T>(p, g, nullptr, T(1), DgH))) return rc;
         CUDA_TRY(timed(p, 3, [&] {
-            return launch_bwd_field<T>(a, mst[s], gH, DgH, gml, g_in, s > 0 ? gk + (s - 1) * n3 : nullptr, back[s],
-                                       g_Ms, g_Ku, p->stream);
+            return launch_bwd_field<T>(a, imap, mst[s], g, DgH, gml, g_in, gvb, s > 0 ? wk[s - 1] : T(0), back[s],
+                                       s > 0 ? mst[s - 1] : nullptr, s > 0 ? Hs + (s - 1) * n3 : nullptr,
+                                       gH[(s & 1) ^ 1], g_Ms, g_Ku, p->stream);
         }));
     }
     return BORIS_OK;

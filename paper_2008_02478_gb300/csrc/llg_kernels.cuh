@@ -92,14 +92,15 @@ template <typename T>
 cudaError_t launch_fwd_stage(const LLGArgs<T>& a, int s, const T* ms, const T* Hd, const T* m0, T* Hs, T* ks,
                              T* mnext, cudaStream_t st);
 template <typename T>
-cudaError_t launch_bwd_start(const LLGArgs<T>& a, const T* m0, const T* k1, const T* k2, const T* k3, const T* k4,
-                             const T* gout, T* gm, T* gk, cudaStream_t st);
+cudaError_t launch_bwd_turn(const LLGArgs<T>& a, const T* m4, const T* Hd, const T* m0, const T* ks, const T* gout, T* gm,
+                            T* gvb, T* gH, T* gml, cudaStream_t st);
+// imap[i] = 1 / (mu0 Ms_i), used by launch_bwd_field with an Ms map;
+// mp, Hp, gHn: state and field of the stage before and the gH it gets; mp NULL at the first stage
 template <typename T>
-cudaError_t launch_bwd_local(const LLGArgs<T>& a, const T* ms, const T* Hs, const T* gk, T* gH, T* gml,
-                             cudaStream_t st);
+cudaError_t launch_bwd_inv_ms(const LLGArgs<T>& a, T* imap, cudaStream_t st);
 template <typename T>
-cudaError_t launch_bwd_field(const LLGArgs<T>& a, const T* ms, const T* gH, const T* DgH, const T* gml, T* gm,
-                             T* gk_prev, T coef, T* gMs, T* gKu, cudaStream_t st);
+cudaError_t launch_bwd_field(const LLGArgs<T>& a, const T* imap, const T* ms, const T* gH, const T* DgH, T* gml, T* gm, const T* gvb, T w,
+                             T coef, const T* mp, const T* Hp, T* gHn, T* gMs, T* gKu, cudaStream_t st);
 struct MLTable;
 cudaError_t launch_rk4_stage_ml(const LLGArgs<float>& a, const MLTable& t, int s, const float* ms, const float* Hd,
                                 float* m0, float* acc, float* mnext, cudaStream_t st);
