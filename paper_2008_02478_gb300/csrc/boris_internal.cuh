@@ -168,8 +168,11 @@ cudaError_t launch_y_4096(const Geometry& g, typename Cx<T>::t* X, typename Cx<T
 // FP32 x complex-to-real (px = 1024, ny even) with the half-spectrum block
 // fetched by tensor copies; a wait that gives up latches BORIS_ERR_TIMEOUT in *status
 bool x_c2r_tma_ok(const Geometry& g, int max_smem);
+// (planes: a multi-mesh frame's, with the most rows of any plane)
+struct MLPlane;
 cudaError_t launch_x_c2r_1024_tma(const Geometry& g, const float2* X, float* H, const float2* tw, int* status,
-                                  unsigned long long limit_ns, cudaStream_t st);
+                                  unsigned long long limit_ns, cudaStream_t st, const MLPlane* planes = nullptr,
+                                  int rows = 0);
 // Tensor-core (FP16 / BF16) z stage of the split schedule (zconv_tc.cu), pz = 64.
 bool zconv_tc_supported(const Geometry& g);
 // bulk-copy pipelined z convolution of the split schedule (FP32; zconv_tma.cu);

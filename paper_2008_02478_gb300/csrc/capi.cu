@@ -124,6 +124,8 @@ struct boris_plan_s {
     unsigned* d_pcode = nullptr;  // [Z * Z] spectrum row offsets / 32, kz sign in bit 31
     float* d_invhz = nullptr;     // [Z] 1 / z size of each plane
     int ml_variant = 1;           // inter-plane sum kernel (ml_mix), chosen by timing at plan time
+    MLMixed mlx = {};       // passes on mixed-radix lengths (planes NULL: the power-of-two frame)
+    MLPlane* d_mlplanes = nullptr;
     float* Mf = nullptr;    // frame fields [3][Z][NY][NX]
     float* Hf = nullptr;
     int ml_unique = 0;
@@ -296,6 +298,35 @@ int ml_demag_apply(boris_plan p, const float* M, const float* ms_map, float ms_s
     float2* X = (float2*)p->X;
     float2* Yb = (float2*)p->Y;
     const float2* tw = (const float2*)p->tw;
+    if (p->mlx.planes) {
+        const MLMixed& x = p->mlx;
+        // axes of 1024 points keep the warp-held transforms (one trip through shared
+        // memory), restricted to the rows that exist; the x inverse copies blocks
+        // that start at even rows of even planes
+        const bool x1024 = p->g.px == 1024, y1024 = p->g.py == 1024, xi1024 = x1024 && x_c2r_tma_ok(p->g, 227 * 1024);
+        CUDA_TRY(timed(p, 0, [&] {
+            if (x1024) return launch_ml_x_r2c_1024(p->g, x.planes, x.rows, M, ms_map, ms_scale, X, tw, p->stream);
+            return launch_ml_x_fwd(x, M, ms_map, ms_scale, X, p->stream);
+        }));
+        auto y_pass = [&](bool fwd) {
+            return timed(p, fwd ? 5 : 7, [&] {
+                if (y1024) return launch_ml_y_1024(p->g, x.planes, X, Yb, tw, p->stream, fwd);
+                return launch_ml_y(x, X, Yb, p->stream, fwd);
+            });
+        };
+        CUDA_TRY(y_pass(true));
+        CUDA_TRY(timed(p, 6, [&] {
+            return ml_mix(p->g, p->mlt.Z, Yb, (const float*)p->Kml, p->d_pairs, p->d_pcode, p->d_invhz, p->ml_variant,
+                          p->nsm, p->stream);
+        }));
+        CUDA_TRY(y_pass(false));
+        CUDA_TRY(timed(p, 2, [&] {
+            if (xi1024)
+                return launch_x_c2r_1024_tma(p->g, X, H, tw, p->d_status, p->wait_limit_ns, p->stream, x.planes, x.rows);
+            return launch_ml_x_inv(x, X, H, p->stream);
+        }));
+        return BORIS_OK;
+    }
     CUDA_TRY(timed(p, 4, [&] { return ml_embed(p->mlt, M, ms_map, ms_scale, p->Mf, p->stream); }));
     CUDA_TRY(timed(p, 0, [&] { return launch_x_r2c<float>(p->g, p->Mf, nullptr, 1.0f, X, tw, p->stream); }));
     CUDA_TRY(timed(p, 5, [&] { return launch_split<float>(p->g, X, Yb, nullptr, tw, p->stream, 0, 2); }));
@@ -751,6 +782,44 @@ int mixed_setup(boris_plan p)
     CUDA_TRY(build_mixed_spectrum(p->g, m, p->dx, p->dy, p->dz, 40.0, p->K, p->f64, p->stream, p->images));
     if ((rc = dev_alloc(p, &p->X, (size_t)p->g.nkx * 3 * p->g.nz * p->g.ny * esz))) return rc;
     CUDA_TRY(cudaStreamSynchronize(p->stream));
+    return BORIS_OK;
+}
+
+// Tables of a multi-mesh plan on mixed-radix lengths: twiddles, positions, planes.
+int ml_mixed_setup(boris_plan p)
+{
+    MixedPlan& m = p->mlx.m;
+    const int nx = line_tw_entries(m.x), ny = line_tw_entries(m.y);
+    std::vector<double2> tw(nx + ny);
+    line_tw_host(m.x, tw.data());
+    line_tw_host(m.y, tw.data() + nx);
+    std::vector<float2> twf;
+    for (const double2& v : tw) twf.push_back(make_float2((float)v.x, (float)v.y));
+    std::vector<unsigned short> pos(2 * (m.x.H + m.y.H));
+    line_pos_host(m.x, (int)sizeof(float2), pos.data());
+    line_pos_host(m.y, (int)sizeof(float2), pos.data() + 2 * m.x.H);
+    const MLTable& t = p->mlt;
+    std::vector<MLPlane> planes(t.Z);
+    p->mlx.rows = 0;
+    for (int z = 0; z < t.Z; z++) {
+        const int l = t.plane_layer[z], q = z - t.plane0[l];
+        const size_t row = (size_t)t.nx[l] * t.ny[l];
+        planes[z] = MLPlane{t.nx[l], t.ny[l], t.ox[l], t.oy[l], t.off[l] + q * row, row * t.nz[l], t.off[l] / 3 + q * row};
+        p->mlx.rows = std::max(p->mlx.rows, t.ny[l]);
+    }
+    int rc;
+    CUDA_TRY(ml_mixed_prepare(p->mlx));
+    if ((rc = dev_alloc(p, &p->mtw, twf.size() * sizeof(float2)))) return rc;
+    if ((rc = dev_alloc(p, (void**)&p->mpos, pos.size() * sizeof(unsigned short)))) return rc;
+    if ((rc = dev_alloc(p, (void**)&p->d_mlplanes, planes.size() * sizeof(MLPlane)))) return rc;
+    CUDA_TRY(cudaMemcpy(p->mtw, twf.data(), twf.size() * sizeof(float2), cudaMemcpyHostToDevice));
+    CUDA_TRY(cudaMemcpy(p->mpos, pos.data(), pos.size() * sizeof(unsigned short), cudaMemcpyHostToDevice));
+    CUDA_TRY(cudaMemcpy(p->d_mlplanes, planes.data(), planes.size() * sizeof(MLPlane), cudaMemcpyHostToDevice));
+    m.twx = p->mtw;
+    m.twy = (const float2*)p->mtw + nx;
+    m.posx = p->mpos;
+    m.posy = p->mpos + 2 * m.x.H;
+    p->mlx.planes = p->d_mlplanes;
     return BORIS_OK;
 }
 
@@ -1319,20 +1388,39 @@ int boris_multimesh_plan(int n_layers, const int* nxyz, const double* hxyz, cons
     int max_smem = 0;
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
     if (!split_supported<float>(g, max_smem)) return bail(fail(BORIS_ERR_UNSUPPORTED_SIZE, "frame too large"));
-    cudaError_t ce = upload_twiddles_split();
-    if (ce == cudaSuccess) ce = upload_twiddles_fast();
-    if (ce == cudaSuccess) ce = upload_twiddles_res();
-    if (ce != cudaSuccess) return bail(fail(BORIS_ERR_CUDA, "twiddle constants"));
-    if ((rc = upload_plan_twiddles(p, g, false))) return bail(rc);
+    const bool mlmixed = ml_mixed_shape(t.NX, t.NY, Z, max_smem, &p->mlx);
+    cudaError_t ce = cudaSuccess;
+    if (mlmixed) {
+        g.px = 2 * p->mlx.m.x.H;
+        g.py = 2 * p->mlx.m.y.H;
+        g.nkx = p->mlx.m.x.H + 1;
+        g.kyh = p->mlx.m.y.H + 1;
+        if (g.px == 1024 || g.py == 1024) {
+            // tables of the length-1024 passes
+            g.lmax = 1024;
+            g.lglmax = 10;
+            if ((rc = upload_plan_twiddles(p, g, false))) return bail(rc);
+        }
+        p->g = g;
+        if ((rc = ml_mixed_setup(p))) return bail(rc);
+    } else {
+        ce = upload_twiddles_split();
+        if (ce == cudaSuccess) ce = upload_twiddles_fast();
+        if (ce == cudaSuccess) ce = upload_twiddles_res();
+        if (ce != cudaSuccess) return bail(fail(BORIS_ERR_CUDA, "twiddle constants"));
+        if ((rc = upload_plan_twiddles(p, g, false))) return bail(rc);
+    }
     const size_t kbytes = (size_t)p->ml_unique * g.nkx * 6 * ml_kyp(g) * sizeof(float);
     if ((rc = dev_alloc(p, &p->Kml, kbytes))) return bail(rc);
     if ((rc = dev_alloc(p, (void**)&p->d_pairs, h.pairs.size() * sizeof(int)))) return bail(rc);
     cudaMemcpy(p->d_pairs, h.pairs.data(), h.pairs.size() * sizeof(int), cudaMemcpyHostToDevice);
-    ce = ml_build_spectra(h, g, (float*)p->Kml, p->tw64, p->stream);
+    ce = ml_build_spectra(h, g, (float*)p->Kml, p->tw64, p->stream, mlmixed ? &p->mlx : nullptr);
     if (ce != cudaSuccess) return bail(fail(BORIS_ERR_CUDA, std::string("inter-mesh spectra: ") + cudaGetErrorString(ce)));
     const size_t frame = 3 * (size_t)Z * t.NY * t.NX;
-    if ((rc = dev_alloc(p, (void**)&p->Mf, frame * sizeof(float)))) return bail(rc);
-    if ((rc = dev_alloc(p, (void**)&p->Hf, frame * sizeof(float)))) return bail(rc);
+    if (!mlmixed) {
+        if ((rc = dev_alloc(p, (void**)&p->Mf, frame * sizeof(float)))) return bail(rc);
+        if ((rc = dev_alloc(p, (void**)&p->Hf, frame * sizeof(float)))) return bail(rc);
+    }
     if ((rc = dev_alloc(p, &p->X, (size_t)g.nkx * 3 * Z * g.ny * sizeof(float2)))) return bail(rc);
     if ((rc = dev_alloc(p, &p->Y, (size_t)g.nkx * g.py * 3 * Z * sizeof(float2)))) return bail(rc);
     // the persistent inter-plane sum reads 32-bit row offsets (128-byte units)
@@ -1740,7 +1828,7 @@ void boris_plan_destroy(boris_plan p)
 {
     if (!p) return;
     cudaStreamSynchronize(p->stream);
-    void* ptrs[] = {p->mtw, p->mpos, p->d_absmax, p->Y16, p->K16, p->Kml, p->d_pairs, p->d_pcode, p->d_invhz, p->Mf, p->Hf, p->K, p->K2, p->d_step, p->X, p->Y, p->Hd, p->msa, p->msb, p->acc, p->kbuf, p->mtrial, p->d_rkf, p->energy,
+    void* ptrs[] = {p->d_mlplanes, p->mtw, p->mpos, p->d_absmax, p->Y16, p->K16, p->Kml, p->d_pairs, p->d_pcode, p->d_invhz, p->Mf, p->Hf, p->K, p->K2, p->d_step, p->X, p->Y, p->Hd, p->msa, p->msb, p->acc, p->kbuf, p->mtrial, p->d_rkf, p->energy,
                     p->m_dev_e2e, p->bw};
     for (void* q : ptrs)
         if (q) cudaFree(q);

@@ -11,6 +11,7 @@
 
 #include "boris_internal.cuh"
 #include "bulk_async.cuh"
+#include "ml_mixed.cuh"
 #include "warp_fft.cuh"
 
 namespace boris {
@@ -19,12 +20,16 @@ constexpr int REG1025 = 1025;  // per-warp region stride (complex): one pad elem
 
 // x real-to-complex, px = 1024: 16 rows (c, z, y0..y0+15) per CTA; warp w packs
 // row w (real part) and row w + 8 (imaginary part) into one complex line.
-template <typename T>
+// WIN: a multi-mesh frame; the rows are those of the layer of plane z, read
+// from its own array and written to their place in the frame (here and in the
+// kernels below).
+template <typename T, bool WIN = false>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) x_r2c_1024_kernel(Geometry g, const T* __restrict__ M,
                                                          const T* __restrict__ ms_map, T ms_scale,
                                                          typename Cx<T>::t* __restrict__ X,
                                                          const typename Cx<T>::t* __restrict__ tw_g,
-                                                         unsigned* __restrict__ absmax)
+                                                         unsigned* __restrict__ absmax,
+                                                         const MLPlane* __restrict__ planes = nullptr)
 {
     using C = typename Cx<T>::t;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -33,27 +38,40 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) x_r2c_1024_kernel
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int y0 = blockIdx.x * 16, z = blockIdx.y, c = blockIdx.z;
     const int nx = g.nx, ny = g.ny, nz = g.nz;
+    // rows of the field: all of them, or (WIN) the layer's, x shifted by its place
+    int rx = nx, ry = ny, ox = 0, oy = 0;
+    size_t row0 = ((size_t)z * ny) * nx, comp = (size_t)nx * ny * nz, mrow0 = row0;
+    if constexpr (WIN) {
+        const MLPlane q = planes[z];
+        rx = q.nx;
+        ry = q.ny;
+        ox = q.ox;
+        oy = q.oy;
+        row0 = q.off;
+        comp = q.comp;
+        mrow0 = q.moff;
+        if (y0 >= ry) return;
+    }
     load_tw1024(tws, tw_g, g.lmax);
     __syncthreads();
-    const size_t ncell = (size_t)nx * ny * nz;
     const int ya = y0 + warp, yb = y0 + warp + 8;
-    const T* ra = M + c * ncell + ((size_t)z * ny + ya) * nx;
-    const T* rb = M + c * ncell + ((size_t)z * ny + yb) * nx;
-    const T* ma = ms_map ? ms_map + ((size_t)z * ny + ya) * nx : nullptr;
-    const T* mb = ms_map ? ms_map + ((size_t)z * ny + yb) * nx : nullptr;
+    const T* ra = M + c * comp + row0 + (size_t)ya * rx - ox;
+    const T* rb = M + c * comp + row0 + (size_t)yb * rx - ox;
+    const T* ma = ms_map ? ms_map + mrow0 + (size_t)ya * rx - ox : nullptr;
+    const T* mb = ms_map ? ms_map + mrow0 + (size_t)yb * rx - ox : nullptr;
     C v[32];
-    const bool oka = ya < ny, okb = yb < ny;
+    const bool oka = ya < ry, okb = yb < ry;
 #pragma unroll
     for (int a = 0; a < 16; a++) {
         const int x = 32 * a + lane;
-        const bool in = x < nx;
+        const bool in = WIN ? x >= ox && x < ox + rx : x < nx;
         v[a] = C{(in && oka) ? ra[x] : T(0), (in && okb) ? rb[x] : T(0)};
     }
     if (ms_map) {
 #pragma unroll
         for (int a = 0; a < 16; a++) {
             const int x = 32 * a + lane;
-            const bool in = x < nx;
+            const bool in = WIN ? x >= ox && x < ox + rx : x < nx;
             v[a].x *= (in && oka) ? ma[x] : T(0);
             v[a].y *= (in && okb) ? mb[x] : T(0);
         }
@@ -86,8 +104,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) x_r2c_1024_kernel
     // its shared and global addresses advance by fixed strides.
     {
         const int t = threadIdx.x & 15, kx0 = threadIdx.x >> 4;
-        const int y = y0 + t;
-        if (y < ny) {
+        const int y = y0 + t + oy;
+        if (y0 + t < ry) {
             const C* line = reg + (t & 7) * REG1025;
             const size_t xstride = (size_t)3 * nz * ny;  // one kx step in X
             C* dst = X + ((size_t)kx0 * 3 + c) * nz * ny + (size_t)z * ny + y;
@@ -178,10 +196,12 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) x_c2r_1024_kernel
 // *status and returns.
 constexpr size_t XC2R_TMA_SMEM = 1024 + 512 * 128 + 128 + (size_t)TW1024_SLOTS * sizeof(float2) + 16;
 
+template <bool WIN>
 __global__ void __launch_bounds__(256, 3) x_c2r_1024_tma_kernel(const __grid_constant__ CUtensorMap xmap, Geometry g,
                                                                  const float2* __restrict__ X, float* __restrict__ H,
                                                                  const float2* __restrict__ tw_g, int* status,
-                                                                 unsigned long long limit_ns)
+                                                                 unsigned long long limit_ns,
+                                                                 const MLPlane* __restrict__ planes)
 {
     extern __shared__ unsigned char smem_raw[];
     // aligned to 1024 bytes by an offset from the shared array itself, so that the
@@ -193,8 +213,15 @@ __global__ void __launch_bounds__(256, 3) x_c2r_1024_tma_kernel(const __grid_con
     uint64_t* bar = reinterpret_cast<uint64_t*>(base + 512 * 128 + 128 + TW1024_SLOTS * sizeof(float2));
     float2* reg = S;  // per-warp transpose regions once the block is consumed
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int y0 = blockIdx.x * 16, z = blockIdx.y, c = blockIdx.z;
+    int y0 = blockIdx.x * 16;
+    const int z = blockIdx.y, c = blockIdx.z;
     const int nx = g.nx, ny = g.ny, nz = g.nz;
+    MLPlane q = {};
+    if constexpr (WIN) {
+        q = planes[z];
+        y0 += q.oy & ~1;  // an even column: the copies start on 16-byte boundaries
+        if (y0 >= q.oy + q.ny) return;
+    }
     const int x0 = (c * nz + z) * ny + y0;  // column of the block in the [kx][(c, z, y)] view of X
     if (threadIdx.x == 0) {
         mbar_init(bar, 1);
@@ -223,6 +250,8 @@ __global__ void __launch_bounds__(256, 3) x_c2r_1024_tma_kernel(const __grid_con
     const float2* loB = S + lane * 16 + 2 * (wb ^ (lane & 7)) + wl;
     const float2* hiA = S + (1024 - lane) * 16 + 2 * (wa ^ (-lane & 7)) + wl;
     const float2* hiB = S + (1024 - lane) * 16 + 2 * (wb ^ (-lane & 7)) + wl;
+    // (WIN) rows of the block outside the layer hold nothing: read as zero
+    const bool ina = !WIN || (ya >= q.oy && ya < q.oy + q.ny), inb = !WIN || (yb >= q.oy && yb < q.oy + q.ny);
     float2 v[32];
 #pragma unroll
     for (int d = 0; d < 32; d++) {
@@ -248,10 +277,25 @@ __global__ void __launch_bounds__(256, 3) x_c2r_1024_tma_kernel(const __grid_con
             A.y = -A.y;
             B.y = -B.y;
         }
+        if (!ina) A = float2{0.f, 0.f};
+        if (!inb) B = float2{0.f, 0.f};
         v[brev5(d)] = float2{A.x - B.y, A.y + B.x};
     }
     __syncthreads();  // the staging block becomes the warps' transpose tiles
     warp_fft1024_inv(v, reg + warp * REG1025, tws);
+    if constexpr (WIN) {
+        const int ra = ya - q.oy, rb = yb - q.oy;  // rows of the layer
+        float* h = H + q.off + c * q.comp - q.ox;
+#pragma unroll
+        for (int a = 0; a < 16; a++) {
+            const int x = 32 * a + lane;
+            if (x >= q.ox && x < q.ox + q.nx) {
+                if (ra >= 0 && ra < q.ny) h[(size_t)ra * q.nx + x] = v[a].x;
+                if (rb >= 0 && rb < q.ny) h[(size_t)rb * q.nx + x] = v[a].y;
+            }
+        }
+        return;
+    }
     const size_t ncell = (size_t)nx * ny * nz;
     float* ha = H + c * ncell + ((size_t)z * ny + ya) * nx;
     float* hb = H + c * ncell + ((size_t)z * ny + yb) * nx;
@@ -288,15 +332,23 @@ bool x_c2r_tma_ok(const Geometry& g, int max_smem)
 }
 
 cudaError_t launch_x_c2r_1024_tma(const Geometry& g, const float2* X, float* H, const float2* tw, int* status,
-                                  unsigned long long limit_ns, cudaStream_t st)
+                                  unsigned long long limit_ns, cudaStream_t st, const MLPlane* planes, int rows)
 {
     CUtensorMap map;
     cudaError_t e = xc2r_map(g, X, &map);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(x_c2r_1024_tma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)XC2R_TMA_SMEM);
+    if (planes) {
+        e = cudaFuncSetAttribute(x_c2r_1024_tma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)XC2R_TMA_SMEM);
+        if (e != cudaSuccess) return e;
+        // one row more than the most of any layer: tiles start at even rows
+        x_c2r_1024_tma_kernel<true><<<dim3((rows + 16) / 16, g.nz, 3), 256, XC2R_TMA_SMEM, st>>>(map, g, X, H, tw, status,
+                                                                                                 limit_ns, planes);
+        return cudaGetLastError();
+    }
+    e = cudaFuncSetAttribute(x_c2r_1024_tma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)XC2R_TMA_SMEM);
     if (e != cudaSuccess) return e;
-    x_c2r_1024_tma_kernel<<<dim3((g.ny + 15) / 16, g.nz, 3), 256, XC2R_TMA_SMEM, st>>>(map, g, X, H, tw, status,
-                                                                                       limit_ns);
+    x_c2r_1024_tma_kernel<false><<<dim3((g.ny + 15) / 16, g.nz, 3), 256, XC2R_TMA_SMEM, st>>>(map, g, X, H, tw, status,
+                                                                                              limit_ns, nullptr);
     return cudaGetLastError();
 }
 
@@ -304,10 +356,11 @@ cudaError_t launch_x_c2r_1024_tma(const Geometry& g, const float2* X, float* H, 
 // Two CTAs per SM (93 registers): 0.099 ms at 512 x 512 x 32 against 0.107 ms
 // with three (80 registers) - fewer lines in flight, and more loads in flight
 // per line; the x passes and the 16-bit y passes measured slower with two.
-template <typename T>
+template <typename T, bool WIN = false>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) y_fwd_1024_kernel(Geometry g, const typename Cx<T>::t* __restrict__ X,
                                                          typename Cx<T>::t* __restrict__ Y,
-                                                         const typename Cx<T>::t* __restrict__ tw_g)
+                                                         const typename Cx<T>::t* __restrict__ tw_g,
+                                                         const MLPlane* __restrict__ planes = nullptr)
 {
     using C = typename Cx<T>::t;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -320,11 +373,17 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) y_fwd_1024_kernel
     __syncthreads();
     if (line >= lines) return;
     const C* src = X + ((size_t)kx * lines + line) * ny;
+    int lo = 0, hi = ny;
+    if constexpr (WIN) {
+        const MLPlane* q = planes + line % g.nz;
+        lo = q->oy;
+        hi = lo + q->ny;
+    }
     C v[32];
 #pragma unroll
     for (int a = 0; a < 32; a++) {
         const int y = 32 * a + lane;
-        v[a] = (a < 16 && y < ny) ? src[y] : C{T(0), T(0)};
+        v[a] = (a < 16 && (!WIN || y >= lo) && y < hi) ? src[y] : C{T(0), T(0)};
     }
     warp_fft1024_fwd<C, true>(v, reg + warp * REG1025, tws);
     C* dst = Y + ((size_t)kx * lines + line) * 1024;
@@ -336,10 +395,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) y_fwd_1024_kernel
 // Its twiddles use the padded-index table layout (measured 0.105 ms against
 // 0.127-0.129 ms with the row-per-c layout at 512 x 512 x 32; the persistent
 // 16-bit inverse below is the other way round).
-template <typename T>
+template <typename T, bool WIN = false>
 __global__ void __launch_bounds__(256) y_inv_1024_kernel(Geometry g, const typename Cx<T>::t* __restrict__ Y,
                                                          typename Cx<T>::t* __restrict__ X,
-                                                         const typename Cx<T>::t* __restrict__ tw_g)
+                                                         const typename Cx<T>::t* __restrict__ tw_g,
+                                                         const MLPlane* __restrict__ planes = nullptr)
 {
     using C = typename Cx<T>::t;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -357,10 +417,16 @@ __global__ void __launch_bounds__(256) y_inv_1024_kernel(Geometry g, const typen
     for (int d = 0; d < 32; d++) v[brev5(d)] = src[lane + 32 * d];
     warp_fft1024_inv<C, false>(v, reg + warp * REG1025, tws);
     C* dst = X + ((size_t)kx * lines + line) * ny;
+    int lo = 0, hi = ny;
+    if constexpr (WIN) {
+        const MLPlane* q = planes + line % g.nz;
+        lo = q->oy;
+        hi = lo + q->ny;
+    }
 #pragma unroll
     for (int a = 0; a < 16; a++) {
         const int y = 32 * a + lane;
-        if (y < ny) dst[y] = v[a];
+        if ((!WIN || y >= lo) && y < hi) dst[y] = v[a];
     }
 }
 
@@ -642,6 +708,35 @@ cudaError_t launch_x_c2r_1024(const Geometry& g, const typename Cx<T>::t* X, T* 
     x_c2r_1024_kernel<T><<<dim3((g.ny + 15) / 16, g.nz, 3), 256, smem, st>>>(g, X, H, tw);
     return cudaGetLastError();
 }
+// The same passes on a multi-mesh frame (px = 1024 / py = 1024, FP32): rows of
+// the layers only.  rows: the most of any plane.
+cudaError_t launch_ml_x_r2c_1024(const Geometry& g, const MLPlane* planes, int rows, const float* M, const float* ms_map,
+                                 float ms, float2* X, const float2* tw, cudaStream_t st)
+{
+    const size_t smem = smem_1024<float>();
+    cudaError_t e = cudaFuncSetAttribute(x_r2c_1024_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    x_r2c_1024_kernel<float, true><<<dim3((rows + 15) / 16, g.nz, 3), 256, smem, st>>>(g, M, ms_map, ms, X, tw, nullptr, planes);
+    return cudaGetLastError();
+}
+cudaError_t launch_ml_y_1024(const Geometry& g, const MLPlane* planes, float2* X, float2* Y, const float2* tw, cudaStream_t st,
+                             bool forward)
+{
+    const size_t smem = smem_1024<float>();
+    const dim3 grid((3 * g.nz + 7) / 8, g.nkx);
+    cudaError_t e;
+    if (forward) {
+        e = cudaFuncSetAttribute(y_fwd_1024_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        y_fwd_1024_kernel<float, true><<<grid, 256, smem, st>>>(g, X, Y, tw, planes);
+    } else {
+        e = cudaFuncSetAttribute(y_inv_1024_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        y_inv_1024_kernel<float, true><<<grid, 256, smem, st>>>(g, Y, X, tw, planes);
+    }
+    return cudaGetLastError();
+}
+
 // The persistent 16-bit y passes apply to even ny and 16-byte aligned arrays;
 // BORIS_Y_PERSIST=0 selects the one-line-per-warp grid instead.
 static bool y_persist_ok(const Geometry& g, const void* a, const void* b)

@@ -16,6 +16,8 @@
 #include "llg_cell.cuh"
 #include "multilayer.cuh"
 
+#include <algorithm>
+
 namespace boris {
 
 // Stage S in 0..3; ms = stage state (m0 itself for S = 0).  What the update
@@ -337,43 +339,42 @@ __global__ void __launch_bounds__(256) energy_kernel(LLGArgs<T> a, const T* __re
 // in layer order, each SoA [3][nz][ny][nx]); exchange couples neighbours
 // inside a layer only (Table 1 exchange with Neumann boundaries per mesh).
 // ---------------------------------------------------------------------------
+// Rate k of cell i (x, y, z) of layer l; vi: its places in the concatenated field.
 template <typename T>
 __device__ __forceinline__ void ml_field_and_rhs(const LLGArgs<T>& a, const MLTable& t, const T* __restrict__ ms,
-                                                 const T* __restrict__ Hd, size_t idx, size_t vi[3], T m[3], T k[3])
+                                                 const T* __restrict__ Hd, int l, unsigned i, int x, int y, int z,
+                                                 unsigned base, unsigned n, T m[3], T k[3])
 {
-    int l = 0;
-    while (l + 1 < t.nl && idx >= t.off[l + 1] / 3) l++;
-    const size_t base = t.off[l], cell = idx - base / 3;
     const int nx = t.nx[l], ny = t.ny[l], nz = t.nz[l];
-    const size_t n = (size_t)nx * ny * nz;
-    const int x = (int)(cell % nx), y = (int)((cell / nx) % ny), z = (int)(cell / ((size_t)nx * ny));
-    for (int c = 0; c < 3; c++) vi[c] = base + c * n + cell;
-    m[0] = ms[vi[0]];
-    m[1] = ms[vi[1]];
-    m[2] = ms[vi[2]];
-    T lap[3] = {T(0), T(0), T(0)};
-    auto nb = [&](size_t j, T w) {
-        lap[0] += w * (ms[vi[0] + j - cell] - m[0]);
-        lap[1] += w * (ms[vi[1] + j - cell] - m[1]);
-        lap[2] += w * (ms[vi[2] + j - cell] - m[2]);
-    };
-    const T ihz2 = T(1) / (T(t.hz[l]) * T(t.hz[l]));
-    const size_t sy = nx, sz = (size_t)nx * ny;
-    if (x > 0) nb(cell - 1, a.ihx2);
-    if (x < nx - 1) nb(cell + 1, a.ihx2);
-    if (y > 0) nb(cell - sy, a.ihy2);
-    if (y < ny - 1) nb(cell + sy, a.ihy2);
-    if (z > 0) nb(cell - sz, ihz2);
-    if (z < nz - 1) nb(cell + sz, ihz2);
+    const unsigned sy = nx, sz = (unsigned)nx * ny, idx = base / 3 + i;
+    const unsigned q[6] = {x > 0 ? i - 1 : i,  x < nx - 1 ? i + 1 : i,  y > 0 ? i - sy : i,
+                           y < ny - 1 ? i + sy : i, z > 0 ? i - sz : i, z < nz - 1 ? i + sz : i};
+    T nb[3][6], H[3];
+#pragma unroll
+    for (int c = 0; c < 3; c++) {
+        const T* f = ms + base + c * n;
+        m[c] = f[i];
+        H[c] = Hd[base + c * n + i];
+#pragma unroll
+        for (int d = 0; d < 6; d++) nb[c][d] = f[q[d]];  // a missing neighbour is the cell itself
+    }
     const T Ms = a.ms_map ? a.ms_map[idx] : a.Ms;
     const T Ku = a.ku_map ? a.ku_map[idx] : a.Ku;
-    const T inv = T(1) / (T(MU0_D) * Ms);
+    const T ihz2 = T(1) / (T(t.hz[l]) * T(t.hz[l]));
+    const T inv = inv_mu0_ms(a, Ms);
     const T cex = T(2) * a.A * inv;
     const T me = m[0] * a.e[0] + m[1] * a.e[1] + m[2] * a.e[2];
     const T can = T(2) * Ku * inv * me;
-    T H[3];
 #pragma unroll
-    for (int c = 0; c < 3; c++) H[c] = Hd[vi[c]] + cex * lap[c] + can * a.e[c] + a.Hext[c];
+    for (int c = 0; c < 3; c++) {
+        T lap = a.ihx2 * (nb[c][0] - m[c]);
+        lap += a.ihx2 * (nb[c][1] - m[c]);
+        lap += a.ihy2 * (nb[c][2] - m[c]);
+        lap += a.ihy2 * (nb[c][3] - m[c]);
+        lap += ihz2 * (nb[c][4] - m[c]);
+        lap += ihz2 * (nb[c][5] - m[c]);
+        H[c] += cex * lap + can * a.e[c] + a.Hext[c];
+    }
     if (a.extra) {
         ext_local_field<T>(a, m, inv, H);
         // surface exchange (Eq. 5): the top plane of layer l with the bottom
@@ -396,42 +397,52 @@ __device__ __forceinline__ void ml_field_and_rhs(const LLGArgs<T>& a, const MLTa
             if (z == 0 && l > 0) couple(l - 1, t.nz[l - 1] - 1);
         }
     }
-    const T mxH[3] = {m[1] * H[2] - m[2] * H[1], m[2] * H[0] - m[0] * H[2], m[0] * H[1] - m[1] * H[0]};
-    const T mmH[3] = {m[1] * mxH[2] - m[2] * mxH[1], m[2] * mxH[0] - m[0] * mxH[2], m[0] * mxH[1] - m[1] * mxH[0]};
-#pragma unroll
-    for (int c = 0; c < 3; c++) k[c] = -a.gp * (mxH[c] + a.alpha * mmH[c]);
+    rhs_from_field(a, m, H, k);
 }
 
-__global__ void __launch_bounds__(256) rk4_stage_ml_kernel(LLGArgs<float> a, MLTable t, int s,
-                                                           const float* __restrict__ ms, const float* __restrict__ Hd,
-                                                           float* __restrict__ m0, float* __restrict__ acc,
-                                                           float* __restrict__ mnext)
+// blockIdx.y is the layer.  All loads of a cell issue together, and the layer's
+// extents are the same for the whole block (with a search per cell and loads
+// behind branches: 91 us on the six-layer stack of 2.9 M cells, now 46).
+template <int S>
+__global__ void __launch_bounds__(256) rk4_stage_ml_kernel(LLGArgs<float> a, MLTable t, const float* __restrict__ ms,
+                                                           const float* __restrict__ Hd, float* __restrict__ m0,
+                                                           float* __restrict__ acc, float* __restrict__ mnext)
 {
-    const size_t n = a.ncell;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        size_t vi[3];
-        float m[3], k[3];
-        ml_field_and_rhs(a, t, ms, Hd, i, vi, m, k);
-        if (s == 0) {
+    const int l = blockIdx.y;
+    const unsigned nx = t.nx[l], ny = t.ny[l], n = nx * ny * t.nz[l], base = (unsigned)t.off[l];
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const unsigned row = i / nx;
+        const int x = (int)(i - row * nx), z = (int)(row / ny), y = (int)(row - (unsigned)z * ny);
+        float b[3] = {}, ac[3] = {};
+        if (S > 0) {
 #pragma unroll
             for (int c = 0; c < 3; c++) {
-                acc[vi[c]] = k[c];
-                mnext[vi[c]] = m[c] + 0.5f * a.dt * k[c];
+                b[c] = m0[base + c * n + i];
+                ac[c] = acc[base + c * n + i];
             }
-        } else if (s < 3) {
-            const float cdt = s == 1 ? 0.5f * a.dt : a.dt;
+        }
+        float m[3], k[3];
+        ml_field_and_rhs(a, t, ms, Hd, l, i, x, y, z, base, n, m, k);
+        if (S == 0) {
 #pragma unroll
             for (int c = 0; c < 3; c++) {
-                acc[vi[c]] += 2.f * k[c];
-                mnext[vi[c]] = m0[vi[c]] + cdt * k[c];
+                acc[base + c * n + i] = k[c];
+                mnext[base + c * n + i] = m[c] + 0.5f * a.dt * k[c];
+            }
+        } else if (S < 3) {
+            const float cdt = S == 1 ? 0.5f * a.dt : a.dt;
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                acc[base + c * n + i] = ac[c] + 2.f * k[c];
+                mnext[base + c * n + i] = b[c] + cdt * k[c];
             }
         } else {
             float v[3];
 #pragma unroll
-            for (int c = 0; c < 3; c++) v[c] = m0[vi[c]] + a.dt * (1.f / 6.f) * (acc[vi[c]] + k[c]);
+            for (int c = 0; c < 3; c++) v[c] = b[c] + a.dt * (1.f / 6.f) * (ac[c] + k[c]);
             const float inv = rsqrtf(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
 #pragma unroll
-            for (int c = 0; c < 3; c++) m0[vi[c]] = v[c] * inv;
+            for (int c = 0; c < 3; c++) m0[base + c * n + i] = v[c] * inv;
         }
     }
 }
@@ -439,9 +450,15 @@ __global__ void __launch_bounds__(256) rk4_stage_ml_kernel(LLGArgs<float> a, MLT
 cudaError_t launch_rk4_stage_ml(const LLGArgs<float>& a, const MLTable& t, int s, const float* ms, const float* Hd,
                                 float* m0, float* acc, float* mnext, cudaStream_t st)
 {
-    size_t b = (a.ncell + 255) / 256;
-    if (b > 152 * 16) b = 152 * 16;
-    rk4_stage_ml_kernel<<<(int)(b > 0 ? b : 1), 256, 0, st>>>(a, t, s, ms, Hd, m0, acc, mnext);
+    size_t most = 1;
+    for (int l = 0; l < t.nl; l++) most = std::max(most, (size_t)t.nx[l] * t.ny[l] * t.nz[l]);
+    const dim3 grid((unsigned)std::min<size_t>((most + 255) / 256, 152 * 16), t.nl);
+    switch (s) {
+    case 0: rk4_stage_ml_kernel<0><<<grid, 256, 0, st>>>(a, t, ms, Hd, m0, acc, mnext); break;
+    case 1: rk4_stage_ml_kernel<1><<<grid, 256, 0, st>>>(a, t, ms, Hd, m0, acc, mnext); break;
+    case 2: rk4_stage_ml_kernel<2><<<grid, 256, 0, st>>>(a, t, ms, Hd, m0, acc, mnext); break;
+    default: rk4_stage_ml_kernel<3><<<grid, 256, 0, st>>>(a, t, ms, Hd, m0, acc, mnext); break;
+    }
     return cudaGetLastError();
 }
 

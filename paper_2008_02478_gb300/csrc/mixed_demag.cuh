@@ -76,4 +76,9 @@ int x_lines(const MixedPlan& m, size_t csz);
 cudaError_t build_mixed_spectrum(const Geometry& g, const MixedPlan& m, double dx, double dy, double dz, double rs,
                                  void* K, bool f64, cudaStream_t st, const int* images);
 
+// One FP64 axis pass of the tensor spectra: [ncomp][d2][d1][d0] with the
+// transformed axis of length n -> H + 1 bins (components in the order xx yy zz xy xz yz).
+cudaError_t run_mixed_axis(const LineFFT& f, const void* in, bool real, double2* out, int axis, int d0, int d1, int d2,
+                           int ncomp, const double2* tw, const unsigned short* pos, cudaStream_t st);
+
 }  // namespace boris

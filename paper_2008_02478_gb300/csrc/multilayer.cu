@@ -515,7 +515,8 @@ __global__ void __launch_bounds__(256, 2) ml_mix_v2_kernel(Geometry g, int Z, fl
     }
 }
 
-cudaError_t ml_build_spectra(const MLHost& h, const Geometry& g, float* K, const double2* tw64, cudaStream_t st)
+cudaError_t ml_build_spectra(const MLHost& h, const Geometry& g, float* K, const double2* tw64, cudaStream_t st,
+                             const MLMixed* mixed)
 {
     const int nu = (int)h.ua.size();
     const int NX = g.nx, NY = g.ny;
@@ -525,8 +526,32 @@ cudaError_t ml_build_spectra(const MLHost& h, const Geometry& g, float* K, const
     if (batch > nu) batch = nu;
     double *ua = nullptr, *ub = nullptr, *udz = nullptr, *T = nullptr;
     double2 *A = nullptr, *B = nullptr;
+    // FP64 tables of the mixed-radix axes
+    LineFFT fx = {}, fy = {};
+    std::vector<double2> tw;
+    std::vector<unsigned short> pos;
+    double2* dtw = nullptr;
+    unsigned short* dpos = nullptr;
+    if (mixed) {
+        if (!make_line_fft(mixed->m.x.H, (int)sizeof(double2), false, &fx) || fx.H != mixed->m.x.H ||
+            !make_line_fft(mixed->m.y.H, (int)sizeof(double2), false, &fy) || fy.H != mixed->m.y.H)
+            return cudaErrorInvalidValue;
+        tw.resize(line_tw_entries(fx) + line_tw_entries(fy));
+        line_tw_host(fx, tw.data());
+        line_tw_host(fy, tw.data() + line_tw_entries(fx));
+        pos.resize(2 * (fx.H + fy.H));
+        line_pos_host(fx, (int)sizeof(double2), pos.data());
+        line_pos_host(fy, (int)sizeof(double2), pos.data() + 2 * fx.H);
+    }
     cudaError_t e = cudaSuccess;
     do {
+        if (mixed) {
+            if ((e = cudaMallocAsync((void**)&dtw, tw.size() * sizeof(double2), st)) != cudaSuccess) break;
+            if ((e = cudaMallocAsync((void**)&dpos, pos.size() * sizeof(unsigned short), st)) != cudaSuccess) break;
+            cudaMemcpyAsync(dtw, tw.data(), tw.size() * sizeof(double2), cudaMemcpyHostToDevice, st);
+            cudaMemcpyAsync(dpos, pos.data(), pos.size() * sizeof(unsigned short), cudaMemcpyHostToDevice, st);
+            if ((e = cudaStreamSynchronize(st)) != cudaSuccess) break;  // the host tables end with this call
+        }
         if ((e = cudaMallocAsync((void**)&ua, nu * sizeof(double), st)) != cudaSuccess) break;
         if ((e = cudaMallocAsync((void**)&ub, nu * sizeof(double), st)) != cudaSuccess) break;
         if ((e = cudaMallocAsync((void**)&udz, nu * sizeof(double), st)) != cudaSuccess) break;
@@ -543,8 +568,17 @@ cudaError_t ml_build_spectra(const MLHost& h, const Geometry& g, float* K, const
             ml_tensor_kernel<<<blocks, 256, 0, st>>>(nb, ua + u0, ub + u0, udz + u0, NX, NY, h.hx, h.hy, 40.0, T);
             if ((e = cudaGetLastError()) != cudaSuccess) break;
             // x then y transform of the parity-extended in-plane tables
-            if ((e = run_axis_n(T, true, A, 0, NX, NY, 1, NX, g.px, 6 * nb, tw64, g.lglmax, st)) != cudaSuccess) break;
-            if ((e = run_axis_n(A, false, B, 1, g.nkx, NY, 1, NY, g.py, 6 * nb, tw64, g.lglmax, st)) != cudaSuccess) break;
+            if (mixed) {
+                e = run_mixed_axis(fx, T, true, A, 0, NX, NY, 1, 6 * nb, dtw, dpos, st);
+                if (e == cudaSuccess)
+                    e = run_mixed_axis(fy, A, false, B, 1, g.nkx, NY, 1, 6 * nb, dtw + line_tw_entries(fx),
+                                       dpos + 2 * fx.H, st);
+            } else {
+                e = run_axis_n(T, true, A, 0, NX, NY, 1, NX, g.px, 6 * nb, tw64, g.lglmax, st);
+                if (e == cudaSuccess)
+                    e = run_axis_n(A, false, B, 1, g.nkx, NY, 1, NY, g.py, 6 * nb, tw64, g.lglmax, st);
+            }
+            if (e != cudaSuccess) break;
             const size_t kt = (size_t)nb * g.nkx * g.kyh * 6;
             blocks = (int)std::min<size_t>((kt + 255) / 256, 152 * 64);
             const int kyp = ml_kyp(g);
@@ -555,6 +589,8 @@ cudaError_t ml_build_spectra(const MLHost& h, const Geometry& g, float* K, const
             e = cudaGetLastError();
         }
     } while (0);
+    if (dtw) cudaFreeAsync(dtw, st);
+    if (dpos) cudaFreeAsync(dpos, st);
     if (ua) cudaFreeAsync(ua, st);
     if (ub) cudaFreeAsync(ub, st);
     if (udz) cudaFreeAsync(udz, st);

@@ -316,7 +316,7 @@ cudaError_t build_kernel_spectrum(const Geometry& g, double dx, double dy, doubl
 template <typename L>
 __global__ void __launch_bounds__(256) mixed_axis_kernel(const void* __restrict__ in, bool in_real,
                                                          double2* __restrict__ out, int axis, int d0, int d1, int d2,
-                                                         int NL, const double2* __restrict__ tw,
+                                                         int ncomp, int NL, const double2* __restrict__ tw,
                                                          const unsigned short* __restrict__ pos)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(256) mixed_axis_kernel(const void* __restrict_
     const int n = dims[axis];
     od[axis] = kh;
     const int oa = axis == 0 ? 1 : 0, ob = axis == 2 ? 1 : 2;
-    const long total = 6L * dims[oa] * dims[ob];
+    const long total = (long)ncomp * dims[oa] * dims[ob];
     const long line0 = (long)blockIdx.x * NL;
     const int nl = (int)min((long)NL, total - line0);
     // line -> component and the base offset of its entry 0 in an array of extents e[]
@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(256) mixed_axis_kernel(const void* __restrict_
             double2 v = make_double2(0.0, 0.0);
             const int src = e < n ? e : e > 2 * H - n ? 2 * H - e : -1;
             if (src >= 0) {
-                const double s = e < n ? 1.0 : comp_parity(c, axis);
+                const double s = e < n ? 1.0 : comp_parity(c % 6, axis);
                 if (in_real) v.x = s * reinterpret_cast<const double*>(in)[b + src * is];
                 else {
                     const double2 t = reinterpret_cast<const double2*>(in)[b + src * is];
@@ -393,6 +393,32 @@ __global__ void mixed_finalize_kernel(const double2* __restrict__ S, typename Cx
     }
 }
 
+cudaError_t run_mixed_axis(const LineFFT& f, const void* in, bool real, double2* out, int axis, int d0, int d1, int d2,
+                           int ncomp, const double2* tw, const unsigned short* pos, cudaStream_t st)
+{
+    int NL = 1;
+    while (NL < 16 && (size_t)2 * NL * f.LS * sizeof(double2) <= 72 * 1024) NL *= 2;
+    const size_t smem = (size_t)NL * f.LS * sizeof(double2);
+    const int dims[3] = {d0, d1, d2};
+    const int oa = axis == 0 ? 1 : 0, ob = axis == 2 ? 1 : 2;
+    const long lines = (long)ncomp * dims[oa] * dims[ob];
+    const unsigned blocks = (unsigned)((lines + NL - 1) / NL);
+    cudaError_t e = cudaErrorInvalidValue;
+    switch (f.id) {
+#define X(i, r1, r2, r3, ...)                                                                                          \
+    case i:                                                                                                            \
+        e = cudaFuncSetAttribute(mixed_axis_kernel<Len<r1, r2, r3, __VA_ARGS__>>,                                      \
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);                              \
+        if (e == cudaSuccess)                                                                                          \
+            mixed_axis_kernel<Len<r1, r2, r3, __VA_ARGS__>><<<blocks, 256, smem, st>>>(in, real, out, axis, d0, d1, d2, \
+                                                                                       ncomp, NL, tw, pos);            \
+        break;
+        BORIS_LENGTHS_FINE(X)
+#undef X
+    }
+    return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
 cudaError_t build_mixed_spectrum(const Geometry& g, const MixedPlan& m, double dx, double dy, double dz, double rs,
                                  void* K, bool f64, cudaStream_t st, const int* images)
 {
@@ -432,26 +458,8 @@ cudaError_t build_mixed_spectrum(const Geometry& g, const MixedPlan& m, double d
         if (nn[a] < 2) continue;
         void* next = nullptr;
         if ((e = cudaMallocAsync(&next, elems(a + 1) * sizeof(double2), st)) != cudaSuccess) break;
-        int NL = 1;
-        while (NL < 16 && (size_t)2 * NL * f[a].LS * sizeof(double2) <= 72 * 1024) NL *= 2;
-        const size_t smem = (size_t)NL * f[a].LS * sizeof(double2);
-        const int oa = a == 0 ? 1 : 0, ob = a == 2 ? 1 : 2;
-        const long lines = 6L * dims[a][oa] * dims[a][ob];
-        const unsigned blocks = (unsigned)((lines + NL - 1) / NL);
-        switch (f[a].id) {
-#define X(i, r1, r2, r3, ...)                                                                                              \
-    case i:                                                                                                           \
-        e = cudaFuncSetAttribute(mixed_axis_kernel<Len<r1, r2, r3, __VA_ARGS__>>, cudaFuncAttributeMaxDynamicSharedMemorySize,     \
-                                 96 * 1024);                                                                          \
-        if (e == cudaSuccess)                                                                                         \
-            mixed_axis_kernel<Len<r1, r2, r3, __VA_ARGS__>><<<blocks, 256, smem, st>>>(cur, real, (double2*)next, a, dims[a][0],   \
-                                                                          dims[a][1], dims[a][2], NL, dtw + two[a],   \
-                                                                          dpos + poso[a]);                            \
-        break;
-            BORIS_LENGTHS_FINE(X)
-#undef X
-        }
-        if (e == cudaSuccess) e = cudaGetLastError();
+        e = run_mixed_axis(f[a], cur, real, (double2*)next, a, dims[a][0], dims[a][1], dims[a][2], 6, dtw + two[a],
+                           dpos + poso[a], st);
         cudaFreeAsync(cur, st);
         cur = next;
         real = false;
