@@ -119,7 +119,7 @@ struct boris_plan_s {
     bool ml = false;
     MLTable mlt;
     double ml_zb[ML_MAX_LAYERS] = {};  // z of each layer's lower face (m)
-    void* Kml = nullptr;    // unique inter-plane spectra [u][kx][c][kyp]
+    void* Kml = nullptr;    // unique inter-plane spectra [u][kx][tile][c][32]
     int* d_pairs = nullptr; // [Z * Z]
     unsigned* d_pcode = nullptr;  // [Z * Z] spectrum row offsets / 32, kz sign in bit 31
     float* d_invhz = nullptr;     // [Z] 1 / z size of each plane

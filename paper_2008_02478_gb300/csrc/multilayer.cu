@@ -106,8 +106,9 @@ __global__ void ml_tensor_kernel(int nu, const double* __restrict__ ua, const do
     }
 }
 
-// 2D spectra [6 nu][kyh][nkx] (complex) -> K[u][kx][c][kyp] (component-major,
-// ky' fastest, rows padded to kyp = kyh rounded up to 32 with zeros) with the
+// 2D spectra [6 nu][kyh][nkx] (complex) -> K[u][kx][tile][c][32] (tiles of
+// 32 ky', the last padded with zeros: what the inter-plane sum stages at once is
+// 768 consecutive bytes) with the
 // real part of xx, yy, zz, xy and the imaginary part of xz, yz (odd in exactly
 // one in-plane axis), scaled by -1/(px py).
 __global__ void ml_finalize_kernel(const double2* __restrict__ S, float* __restrict__ K, int nu, int nkx, int kyh,
@@ -116,10 +117,11 @@ __global__ void ml_finalize_kernel(const double2* __restrict__ S, float* __restr
     const size_t per = (size_t)nkx * kyh;
     const size_t total = (size_t)nu * nkx * 6 * kyp;
     for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total; idx += (size_t)gridDim.x * blockDim.x) {
-        const int ky = (int)(idx % kyp);
-        size_t rest = idx / kyp;
+        size_t rest = idx / 32;
         const int c = (int)(rest % 6);
         rest /= 6;
+        const int ky = (int)(rest % (kyp / 32)) * 32 + (int)(idx % 32);
+        rest /= kyp / 32;
         const int kx = (int)(rest % nkx);
         const int u = (int)(rest / nkx);
         float v = 0.f;
@@ -176,7 +178,7 @@ __global__ void ml_extract_kernel(MLTable t, const float* __restrict__ F, float*
 // column ky = ky' and its mirror py - ky' (which read the same spectrum row,
 // with xy and yz negated), so every spectrum entry is loaded once per kx.
 // Warp w accumulates the target planes p = w, w + 8, ...  Y layout
-// [kx][c][p][ky]; K[u][kx][c][kyp] (one coalesced 128-byte load per component);
+// [kx][c][p][ky]; K[u][kx][tile][c][32] (one coalesced 128-byte load per component);
 // pairs[p * Z + q] = u (>= 0) with bit 30 set when z_p < z_q (xz and yz change
 // sign).
 template <int PMAX>
@@ -204,7 +206,7 @@ __global__ void __launch_bounds__(256) ml_mix_kernel(Geometry g, int Z, float2* 
     }
     __syncthreads();
     const size_t ustride = (size_t)g.nkx * 6 * kyp;
-    const float* Kc = K + (size_t)kx * 6 * kyp + (onA ? kf : 0);
+    const float* Kc = K + (size_t)kx * 6 * kyp + (size_t)blockIdx.x * 192 + lane;
     float2 acc[PMAX][2][3];
 #pragma unroll
     for (int j = 0; j < PMAX; j++)
@@ -226,8 +228,8 @@ __global__ void __launch_bounds__(256) ml_mix_kernel(Geometry g, int Z, float2* 
                 const int u = code & 0x3fffffff;
                 const float sz = (code >> 30) & 1 ? -1.f : 1.f;
                 const float* k = Kc + (size_t)u * ustride;
-                const float kxx = k[0], kyy = k[kyp], kzz = k[2 * kyp], kxy0 = k[3 * kyp];
-                const float kxz = sz * k[4 * kyp], kyz0 = sz * k[5 * kyp];  // imaginary parts: i kxz, i kyz
+                const float kxx = k[0], kyy = k[32], kzz = k[64], kxy0 = k[96];
+                const float kxz = sz * k[128], kyz0 = sz * k[160];  // imaginary parts: i kxz, i kyz
 #pragma unroll
                 for (int h = 0; h < 2; h++) {
                     const float kxy = h ? -kxy0 : kxy0, kyz = h ? -kyz0 : kyz0;  // mirror: ky odd entries flip
@@ -288,7 +290,7 @@ __global__ void __launch_bounds__(256, 2) ml_mix_staged_kernel(Geometry g, int Z
     // lane's share of a target's six 128-byte rows: 16-byte part lane & 7 of
     // components lane >> 3 and (lane >> 3) + 4 (the latter for lanes 0..15)
     const int part = lane & 7, c0 = lane >> 3;
-    const float* Kx = K + (size_t)kx * 6 * kyp + kf0 + part * 4;
+    const float* Kx = K + (size_t)kx * 6 * kyp + (size_t)blockIdx.x * 192 + part * 4;
     for (int i = threadIdx.x; i < Z * Z; i += 256) pr[i] = pairs[i];
     __syncthreads();
     auto stage = [&](int q, int b) {
@@ -298,8 +300,8 @@ __global__ void __launch_bounds__(256, 2) ml_mix_staged_kernel(Geometry g, int Z
             if (p < Z) {
                 const float* src = Kx + (size_t)(pr[p * Z + q] & 0x3fffffff) * ustride;
                 float* dst = Kw + ((size_t)(b * nt + j) * 6) * 32 + part * 4;
-                cp_async16(dst + c0 * 32, src + (size_t)c0 * kyp);
-                if (c0 < 2) cp_async16(dst + (c0 + 4) * 32, src + (size_t)(c0 + 4) * kyp);
+                cp_async16(dst + c0 * 32, src + c0 * 32);
+                if (c0 < 2) cp_async16(dst + (c0 + 4) * 32, src + (c0 + 4) * 32);
             }
         }
         cp_async_commit();
@@ -375,120 +377,154 @@ __global__ void __launch_bounds__(256, 2) ml_mix_staged_kernel(Geometry g, int Z
 
 // The inter-plane sum as one persistent launch over all work items (kx,
 // 32-column tile of folded ky'), tiles of one kx consecutive.  Per item: the
-// Z planes' 32 columns and their mirrors go to shared memory (the mirror's
-// M_y negated, see below); then for each source plane q every warp stages, by
-// cp.async one source ahead, the 6 x 128-byte spectrum rows of its own
-// targets p = warp + 8 j, whose offsets (in 128-byte units, the kz sign in
-// bit 31) come precomputed in pcode; the 3 x 3 products run as packed FP32x2
-// multiply-adds on (Re, Im) pairs.  The mirror column ky -> py - ky flips the
-// ky-odd entries xy and yz; with M_y negated in the mirror the same entries
-// give the mirror's H_x, H_z and -H_y, so both columns share one set of
-// entry pairs.  The source loop is compiled for the warp's exact target count
-// (the counts of the warps differ by at most one), so it has no per-target
-// branches.
+// Z planes' 32 columns and their mirrors go to shared memory; then for each
+// source plane q every warp stages, by cp.async one source ahead, the 768-byte
+// entry sets of its own targets, Z / 8 consecutive planes, and the 3 x 3
+// products run as packed FP32x2 multiply-adds on (Re, Im) pairs.  The mirror
+// column ky -> py - ky flips the ky-odd entries xy and yz; with M_y negated in
+// the mirror the same entries give the mirror's H_x, H_z and -H_y, so both
+// columns share one set of entry pairs.
+//
+// Instruction issue bounds it, so what is not a product is kept out of the
+// source loop: the sets' offsets are listed per warp in the order of use; each
+// set is one piece per lane and a predicated one for half of them; the kz sign
+// goes to the source column (i M, which only the kz-odd entries multiply) where
+// all of a warp's targets are on one side of the source, which consecutive
+// targets make the rule; and the loop is compiled for the warp's exact target
+// count (the counts differ by at most one).  On 34 planes of 512 x 512 (2.0 GB of
+// spectra, 0.86 GB of columns read and written) 1030 -> 833 us; on 32 planes of
+// 200 x 200 131 M warp instructions (66 per target and source) became 102 M, half
+// of the issue slots, 56 % of the shared-memory cycles, 43 % of the multiply-add
+// pipe.  One set for both directions of a pair of planes (8 or 12 warps with
+// their own columns and sums in registers, the other side's through shared
+// memory) fetched 0.63 of the sets and was no faster: 1000-1100 us.
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-
-template <int NT, int PM>
-__device__ __forceinline__ void ml_v2_sum(int Z, int warp, int lane, const float* __restrict__ Kx, int kyp, float* Kw,
-                                          const float2* Ms, const unsigned* pc, float2 (&acc)[PM][2][3])
+// 16 bytes per lane where on (a predicate, not a branch)
+__device__ __forceinline__ void cp_async16_if(void* dst, const void* src, bool on)
 {
-    // the NT targets' 6 rows x 8 sixteen-byte pieces of source q into buffer b:
-    // lane (c0 = lane / 8, part = lane mod 8) copies piece part of rows c0 and,
-    // for c0 < 2, c0 + 4 of each target
-    const int part = lane & 7, c0 = lane >> 3;
-    const int so0 = c0 * kyp + part * 4, so1 = (c0 + 4) * kyp + part * 4;
-    const int do0 = c0 * 32 + part * 4, do1 = (c0 + 4) * 32 + part * 4;
-    // the kz signs of the staged source: bit j = bit 31 of target j's code
-    unsigned sgm = 0, sgm_next = 0;
-    auto stage = [&](int q, int b, unsigned& sgbits) {
-        float* dstb = Kw + (size_t)b * NT * 6 * 32;
-        sgbits = 0;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p cp.async.cg.shared.global [%0], [%1], 16;\n\t}" ::"r"(
+                     smem_u32(dst)),
+                 "l"(src), "r"((int)on)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async8_zfill(void* dst, const void* src, bool ok)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(ok ? 8 : 0) : "memory");
+}
+
+// entry sets of source q (seq: the NT targets' offsets) into slot b of the warp's ring; src, dst at the lane's piece
+template <int NT>
+__device__ __forceinline__ void ml_v2_stage(const unsigned* seq, const float* src, float* dst, bool two, int q, int b)
+{
 #pragma unroll
-        for (int j = 0; j < NT; j++) {
-            const unsigned code = pc[(warp + 8 * j) * Z + q];
-            sgbits |= (code >> 31) << j;
-            const float* src = Kx + (size_t)(code & 0x7fffffffu) * 32;
-            cp_async16(dstb + j * 6 * 32 + do0, src + so0);
-            if (c0 < 2) cp_async16(dstb + j * 6 * 32 + do1, src + so1);
+    for (int j = 0; j < NT; j++) {
+        const float* k = src + (size_t)seq[q * NT + j] * 32;
+        float* d = dst + (b * NT + j) * 192;
+        cp_async16(d, k);
+        cp_async16_if(d + 128, k + 128, two);
+    }
+    cp_async_commit();
+}
+
+// MIXED: the sign differs between the targets (bit j of sg)
+template <int NT, int PM, bool MIXED>
+__device__ __forceinline__ void ml_v2_products(const float* kb, const float2 (&m)[2][3], const float2 (&im)[2][3], unsigned sg,
+                                               float2 (&acc)[PM][2][3])
+{
+#pragma unroll
+    for (int j = 0; j < NT; j++) {
+        const float* k = kb + j * 192;
+        float xz = k[128], yz = k[160];
+        if (MIXED) {
+            const unsigned sb = (sg << (31 - j)) & 0x80000000u;
+            xz = __uint_as_float(__float_as_uint(xz) ^ sb);
+            yz = __uint_as_float(__float_as_uint(yz) ^ sb);
         }
-        cp_async_commit();
-    };
-    stage(0, 0, sgm);
-    for (int q = 0; q < Z; q++) {
-        if (q + 1 < Z) {
-            stage(q + 1, (q + 1) & 1, sgm_next);
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
+        const float2 bxx = f2(k[0]), byy = f2(k[32]), bzz = f2(k[64]), bxy = f2(k[96]), bxz = f2(xz), byz = f2(yz);
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            acc[j][h][0] = ffma2(bxx, m[h][0], ffma2(bxy, m[h][1], ffma2(bxz, im[h][2], acc[j][h][0])));
+            acc[j][h][1] = ffma2(bxy, m[h][0], ffma2(byy, m[h][1], ffma2(byz, im[h][2], acc[j][h][1])));
+            acc[j][h][2] = ffma2(bxz, im[h][0], ffma2(byz, im[h][1], ffma2(bzz, m[h][2], acc[j][h][2])));
         }
+    }
+}
+
+// Sums over the sources; source 0's sets are on their way into slot b, and those
+// of the next item's (at next) when it returns.
+template <int NT, int PM>
+__device__ __forceinline__ void ml_v2_sum(int Z, int lane, const float* src, const float* next, float* ring, int b,
+                                          const float2* Ms, const unsigned* seq, const unsigned char* sgn, float2 (&acc)[PM][2][3])
+{
+    const bool two = lane < 16;
+#pragma unroll 1
+    for (int q = 0; q < Z; q++, b ^= 1) {
+        const bool last = q + 1 == Z;
+        ml_v2_stage<NT>(seq, last ? next : src, ring + lane * 4, two, last ? 0 : q + 1, b ^ 1);
+        cp_async_wait<1>();
         __syncwarp();  // every lane's copies of source q are visible to the warp
-        const float* kb = Kw + (size_t)(q & 1) * NT * 6 * 32 + lane;
+        const float* kb = ring + b * (NT * 192) + lane;
+        const unsigned sg = sgn[q];
+        const bool mixed = sg != 0 && sg != (1u << NT) - 1;
+        const unsigned flip = sg == 0 || mixed ? 0u : 0x80000000u;
         // source columns m and i m (i times, for the imaginary xz and yz entries)
         float2 m[2][3], im[2][3];
 #pragma unroll
         for (int h = 0; h < 2; h++)
 #pragma unroll
             for (int c = 0; c < 3; c++) {
-                m[h][c] = Ms[((q * 3 + c) * 2 + h) * 32 + lane];
-                im[h][c] = make_float2(-m[h][c].y, m[h][c].x);
+                m[h][c] = Ms[((c * Z + q) * 2 + h) * 32 + lane];
+                if (h && c == 1) m[h][c] = make_float2(-m[h][c].x, -m[h][c].y);  // the mirror's M_y, negated
+                im[h][c] = make_float2(__uint_as_float(__float_as_uint(-m[h][c].y) ^ flip),
+                                       __uint_as_float(__float_as_uint(m[h][c].x) ^ flip));
             }
-#pragma unroll
-        for (int j = 0; j < NT; j++) {
-            const float* k = kb + j * 6 * 32;
-            // the kz-odd entries change sign for a source above the target
-            const unsigned sg = ((sgm >> j) & 1u) << 31;
-            const float2 bxx = f2(k[0]), byy = f2(k[32]), bzz = f2(k[64]), bxy = f2(k[96]);
-            const float2 bxz = f2(__uint_as_float(__float_as_uint(k[128]) ^ sg));
-            const float2 byz = f2(__uint_as_float(__float_as_uint(k[160]) ^ sg));
-#pragma unroll
-            for (int h = 0; h < 2; h++) {
-                acc[j][h][0] = ffma2(bxx, m[h][0], ffma2(bxy, m[h][1], ffma2(bxz, im[h][2], acc[j][h][0])));
-                acc[j][h][1] = ffma2(bxy, m[h][0], ffma2(byy, m[h][1], ffma2(byz, im[h][2], acc[j][h][1])));
-                acc[j][h][2] = ffma2(bxz, im[h][0], ffma2(byz, im[h][1], ffma2(bzz, m[h][2], acc[j][h][2])));
-            }
-        }
-        __syncwarp();  // buffer q & 1 is free for source q + 2
-        sgm = sgm_next;
+        if (mixed) ml_v2_products<NT, PM, true>(kb, m, im, sg, acc);
+        else ml_v2_products<NT, PM, false>(kb, m, im, sg, acc);
+        __syncwarp();  // slot b is free for source q + 2
     }
 }
 
 template <int PMAX>
 __global__ void __launch_bounds__(256, 2) ml_mix_v2_kernel(Geometry g, int Z, float2* __restrict__ Y,
-                                                           const float* __restrict__ K, int kyp,
+                                                           const float* __restrict__ K,
                                                            const unsigned* __restrict__ pcode,
                                                            const float* __restrict__ inv_hz, int ntile, int nwork)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nt = (Z - warp + 7) / 8;
-    int before = 0;
-    for (int v = 0; v < warp; v++) before += (Z - v + 7) / 8;
-    float* Kw = reinterpret_cast<float*>(smem_raw) + (size_t)before * 2 * 6 * 32;
-    float2* Ms = reinterpret_cast<float2*>(reinterpret_cast<float*>(smem_raw) + (size_t)Z * 2 * 6 * 32);
-    unsigned* pc = reinterpret_cast<unsigned*>(Ms + (size_t)Z * 3 * 64);
-    float* ih = reinterpret_cast<float*>(pc + (size_t)Z * Z);
-    const int py = g.py;
-    for (int i = threadIdx.x; i < Z * Z; i += 256) pc[i] = pcode[i];
-    for (int i = threadIdx.x; i < Z; i += 256) ih[i] = inv_hz[i];
-    __syncthreads();
+    constexpr int NL = PMAX > 1 ? PMAX - 1 : 0;  // targets of the other warps
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, py = g.py;
+    const int p0 = warp * Z / 8, nt = (warp + 1) * Z / 8 - p0;
+    float* ring = reinterpret_cast<float*>(smem_raw) + (size_t)p0 * 2 * 192;  // [2][nt][6][32]
+    float2* Ms = reinterpret_cast<float2*>(reinterpret_cast<float*>(smem_raw) + (size_t)Z * 2 * 192);  // [c][plane][half][32]
+    unsigned* seq = reinterpret_cast<unsigned*>(Ms + (size_t)Z * 3 * 64) + p0 * Z;                     // [source][nt]
+    unsigned char* sgn = reinterpret_cast<unsigned char*>(reinterpret_cast<unsigned*>(Ms + (size_t)Z * 3 * 64) + Z * Z) + warp * Z;
+    for (int i = lane; i < nt * Z; i += 32) seq[i] = pcode[(p0 + i % nt) * Z + i / nt] & 0x7fffffffu;
+    for (int q = lane; q < Z; q += 32) {
+        unsigned m = 0;
+        for (int j = 0; j < nt; j++) m |= (pcode[(p0 + j) * Z + q] >> 31) << j;
+        sgn[q] = (unsigned char)m;
+    }
+    __syncwarp();
+    const float* Kl = K + lane * 4;
+    if (nt == PMAX) ml_v2_stage<PMAX>(seq, Kl + (size_t)blockIdx.x * 192, ring + lane * 4, lane < 16, 0, 0);
+    else ml_v2_stage<NL>(seq, Kl + (size_t)blockIdx.x * 192, ring + lane * 4, lane < 16, 0, 0);
+    int b = 0;
     for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
         const int kx = w / ntile, kf0 = (w - kx * ntile) * 32;
         const int kf = kf0 + lane;
         const bool onA = kf <= py / 2;
         const bool onB = kf > 0 && kf < py / 2;
         float2* base = Y + (size_t)kx * 3 * Z * py;
-        const float* Kx = K + (size_t)kx * 6 * kyp + kf0;
+        const int wn = w + gridDim.x < nwork ? w + gridDim.x : w;  // (the last item's first sets once more)
+        const float *src = Kl + (size_t)w * 192, *next = Kl + (size_t)wn * 192;  // items are in the set's order
         for (int i = threadIdx.x; i < 3 * Z * 64; i += 256) {
-            const int col = i & 31, half = (i >> 5) & 1, line = i >> 6;  // line = c * Z + p
-            const int c = line / Z, p = line - c * Z;
-            const int f = kf0 + col;
+            const int half = (i >> 5) & 1, line = i >> 6, f = kf0 + (i & 31);
             const bool ok = half ? (f > 0 && f < py / 2) : (f <= py / 2);
-            const int ky = half ? py - f : f;
-            float2 v = ok ? base[(size_t)line * py + ky] : make_float2(0.f, 0.f);
-            if (half && c == 1) v = make_float2(-v.x, -v.y);  // the mirror's M_y, negated
-            Ms[((p * 3 + c) * 2 + half) * 32 + col] = v;
+            cp_async8_zfill(Ms + i, base + (size_t)line * py + (ok ? (half ? py - f : f) : 0), ok);
         }
+        cp_async_commit();
+        cp_async_wait<0>();
         __syncthreads();  // the columns are in shared memory
         float2 acc[PMAX][2][3];
 #pragma unroll
@@ -497,13 +533,13 @@ __global__ void __launch_bounds__(256, 2) ml_mix_v2_kernel(Geometry g, int Z, fl
             for (int h = 0; h < 2; h++)
 #pragma unroll
                 for (int c = 0; c < 3; c++) acc[j][h][c] = make_float2(0.f, 0.f);
-        if (nt == PMAX) ml_v2_sum<PMAX, PMAX>(Z, warp, lane, Kx, kyp, Kw, Ms, pc, acc);
-        else if (nt == PMAX - 1) ml_v2_sum<(PMAX > 1 ? PMAX - 1 : 0), PMAX>(Z, warp, lane, Kx, kyp, Kw, Ms, pc, acc);
+        if (nt == PMAX) ml_v2_sum<PMAX, PMAX>(Z, lane, src, next, ring, b, Ms, seq, sgn, acc);
+        else ml_v2_sum<NL, PMAX>(Z, lane, src, next, ring, b, Ms, seq, sgn, acc);
 #pragma unroll
         for (int j = 0; j < PMAX; j++) {
-            const int p = warp + 8 * j;
-            if (p < Z) {
-                const float ia = ih[p];  // the spectra hold a N: divide by the target's a
+            if (j < nt) {
+                const int p = p0 + j;
+                const float ia = inv_hz[p];  // the spectra hold a N: divide by the target's a
 #pragma unroll
                 for (int c = 0; c < 3; c++) {
                     if (onA) base[(size_t)(c * Z + p) * py + kf] = __fmul2_rn(acc[j][0][c], f2(ia));
@@ -511,8 +547,10 @@ __global__ void __launch_bounds__(256, 2) ml_mix_v2_kernel(Geometry g, int Z, fl
                 }
             }
         }
+        b ^= Z & 1;
         __syncthreads();  // the column stage is reused by the next item
     }
+    cp_async_wait<0>();
 }
 
 cudaError_t ml_build_spectra(const MLHost& h, const Geometry& g, float* K, const double2* tw64, cudaStream_t st,
@@ -625,7 +663,7 @@ int ml_kyp(const Geometry& g) { return (g.kyh + 31) / 32 * 32; }
 size_t ml_mix_v2_smem(int Z)
 {
     return (size_t)Z * 2 * 6 * 32 * sizeof(float) + (size_t)Z * 3 * 64 * sizeof(float2) +
-           (size_t)Z * Z * sizeof(unsigned) + (size_t)Z * sizeof(float);
+           (size_t)Z * Z * sizeof(unsigned) + (size_t)8 * Z;
 }
 
 cudaError_t ml_mix(const Geometry& g, int Z, float2* Y, const float* K, const int* pairs, const unsigned* pcode,
@@ -643,7 +681,7 @@ cudaError_t ml_mix(const Geometry& g, int Z, float2* Y, const float* K, const in
 #define ML_V2(P)                                                                                             \
     e = cudaFuncSetAttribute(ml_mix_v2_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);   \
     if (e != cudaSuccess) return e;                                                                          \
-    ml_mix_v2_kernel<P><<<G, 256, smem, st>>>(g, Z, Y, K, kyp, pcode, inv_hz, ntile, nwork);                 \
+    ml_mix_v2_kernel<P><<<G, 256, smem, st>>>(g, Z, Y, K, pcode, inv_hz, ntile, nwork);                      \
     return cudaGetLastError();
         if (pmax <= 1) { ML_V2(1) }
         if (pmax <= 2) { ML_V2(2) }
@@ -651,6 +689,7 @@ cudaError_t ml_mix(const Geometry& g, int Z, float2* Y, const float* K, const in
         if (pmax <= 4) { ML_V2(4) }
         if (pmax <= 5) { ML_V2(5) }
         if (pmax <= 6) { ML_V2(6) }
+        if (pmax <= 7) { ML_V2(7) }
         if (pmax <= 8) { ML_V2(8) }
 #undef ML_V2
         return cudaErrorInvalidValue;

@@ -50,7 +50,7 @@ cudaError_t ml_extract(const MLTable& t, const float* F, float* H, cudaStream_t 
 cudaError_t ml_mix(const Geometry& g, int Z, float2* Y, const float* K, const int* pairs, const unsigned* pcode,
                    const float* inv_hz, int variant, int nsm, cudaStream_t st);
 size_t ml_mix_v2_smem(int Z);
-// row pitch of the multi-mesh spectra K[u][kx][c][kyp]
+// ky' entries of the multi-mesh spectra K[u][kx][tile][c][32], tiles included
 int ml_kyp(const Geometry& g);
 
 }  // namespace boris

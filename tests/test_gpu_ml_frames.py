@@ -80,3 +80,24 @@ def test_frames_with_a_magnetisation_map(layers):
     assert dt * 2.22e5 * np.abs(H).max() < 2e-3
     ref = dt * llg.llg_rhs(m0.T, H.T, llg.Params(cell=(1, 1, 1), alpha=0.1)).T
     assert rel_l2(m1 - m0, ref) < 2e-3
+
+
+PLANES = [[1], [1, 2], [3, 4], [8], [4, 4, 1], [6, 6, 4], [10, 7], [16, 8, 1], [14, 20], [24, 16], [20, 1, 20], [16, 16, 16], [49]]
+
+
+@pytest.mark.parametrize("planes", PLANES)
+@pytest.mark.parametrize("ny,variant", [(5, 2), (5, 3), (35, 2)])
+def test_persistent_sum_over_plane_counts(planes, ny, variant, monkeypatch):
+    """The persistent inter-plane sum over its plane counts: one plane, fewer
+    than the eight warps, equal and unequal counts of consecutive targets, and
+    sources below, above and between a warp's targets; one and several column
+    tiles.  Sampled cells of the direct sum."""
+    torch = torch_cuda()
+    if variant == 3 and sum(planes) > 36:
+        pytest.skip("two blocks per SM hold 36 planes")
+    monkeypatch.setenv("BORIS_ML_MIX", str(variant))
+    st, m, M, plan = make_case([(5 - l, ny - l, nz) for l, nz in enumerate(planes)])
+    assert plan.schedule()[2] == variant
+    H = plan.apply(torch.tensor(M, dtype=torch.float32, device="cuda")).cpu().numpy()
+    cells, got = sampled(st, H)
+    assert_close(got, ml.direct_at(st, M, cells), 1e-5)
