@@ -188,7 +188,7 @@ int boris_demag_apply_f64(boris_plan p, const double* M, double* Hd);
  *   GPU that loads the library until the process exits), so it accepts meshes
  *   whose spectral workspace - (px/2 + 1) * 3 * nz * ny * 8 bytes, plus
  *   (px/2 + 1) * py * 3 * nz * 8 bytes when the plan chose the split y-z
- *   schedule (on schedule kind 3: where the split schedule serves the mesh),
+ *   schedule (on kinds 3 and 4: where the split schedule serves the mesh),
  *   px and py powers of two - fits in 32 MiB, and returns BORIS_ERR_UNSUPPORTED_SIZE for
  *   larger ones.  The plan (made at set-up)
  *   still supplies the kernel spectrum.  The plan's device must be current.
@@ -399,20 +399,21 @@ int boris_sync_status(boris_plan p);
 const char* boris_last_error(void);
 
 /* Padded transform lengths chosen by the plan: out[0..2] = px, py, pz (powers
- * of two, or on schedule kind 3 twice the smallest half length of its mixed-
- * radix set that holds the axis). */
+ * of two, or on schedule kinds 3 and 4 twice the smallest half length of their
+ * mixed-radix set that holds the axis; multi-mesh frames likewise). */
 int boris_plan_padded(boris_plan p, int out[3]);
 
 /* Schedule of the y-z pass chosen by the plan's autotuner (CUDA-event
  * timing of every candidate that fits the mesh): out[0] kind (0: fused, z
  * stage through shared-memory passes, 1: fused, z stage in registers, 2:
  * split into y-forward / z-convolution / y-inverse kernels, 3: one CTA per kx
- * plane on mixed-radix lengths, taken without timing by a rule on the sizes
- * where a padded plane fits a CTA's shared memory; multi-mesh plans
+ * plane on mixed-radix lengths, where a padded plane fits a CTA's shared
+ * memory, 4: y, z and y passes on mixed-radix lengths (FP32, nz > 1); 3 and 4
+ * are taken without timing by a rule on the sizes; multi-mesh plans
  * report kind 2 with out[2] the inter-plane sum variant: 0 one CTA per tile,
  * 1 staged rows, 2 or 3 one persistent launch with 1 or 2 CTAs per SM).
- * Kinds 0, 1 and 3:
- * out[1] CTAs per cluster (kind 3: 1), out[2] threads per CTA, out[3] shared memory per
+ * Kinds 0, 1, 3 and 4:
+ * out[1] CTAs per cluster (3 and 4: 1), out[2] threads per CTA (4: of the z pass), out[3] shared memory per
  * CTA.  Kind 2: out[1] CTAs per SM the z convolution's register budget is
  * fitted to, out[2] the z-convolution variant: 1 or 2 for the persistent
  * bulk-copy (TMA) pipeline with one or two tile stages, 3 for the residue-
@@ -425,8 +426,8 @@ int boris_plan_padded(boris_plan p, int out[3]);
  * boris_sync_status.
  * Environment overrides read at plan creation restrict the candidates:
  * BORIS_YZ_KIND, BORIS_YZ_CLUSTER, BORIS_YZ_THREADS, BORIS_YZ_QC (kind 0
- * chunk), BORIS_YZ_TMA (kind 2 variant); with any of them set, kind 3 is taken
- * only where BORIS_YZ_KIND=3 asks for it. */
+ * chunk), BORIS_YZ_TMA (kind 2 variant); with any of them set, kinds 3 and 4
+ * are taken only where BORIS_YZ_KIND=3 or 4 asks for them. */
 int boris_plan_schedule(boris_plan p, int out[4]);
 
 /* Bytes of device memory owned by the plan. */

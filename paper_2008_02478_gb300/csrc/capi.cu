@@ -311,7 +311,7 @@ int ml_demag_apply(boris_plan p, const float* M, const float* ms_map, float ms_s
         auto y_pass = [&](bool fwd) {
             return timed(p, fwd ? 5 : 7, [&] {
                 if (y1024) return launch_ml_y_1024(p->g, x.planes, X, Yb, tw, p->stream, fwd);
-                return launch_ml_y(x, X, Yb, p->stream, fwd);
+                return launch_line_y(x.m, x.planes, 3 * x.Z, x.Z, X, Yb, p->stream, fwd);
             });
         };
         CUDA_TRY(y_pass(true));
@@ -351,6 +351,16 @@ int demag_to_spectrum_t(boris_plan p, const T* M, const T* ms_map, T ms_scale)
                 return launch_x_r2c<T>(p->g, M, ms_map, ms_scale, (C*)p->X, (const C*)p->tw, p->stream);
             return launch_mixed_x_fwd<T>(p->mp, M, ms_map, ms_scale, (C*)p->X, p->stream);
         }));
+        if constexpr (sizeof(T) == 4) {
+            if (p->mp.split) {
+                C *X = (C*)p->X, *Y = (C*)p->Y;
+                const C* tw = (const C*)p->tw;
+                CUDA_TRY(timed(p, 5, [&] { return launch_mixed_y(p->mp, p->g, X, Y, tw, p->stream, true); }));
+                CUDA_TRY(timed(p, 6, [&] { return launch_mixed_z(p->mp, Y, (const C*)p->K, p->stream); }));
+                CUDA_TRY(timed(p, 7, [&] { return launch_mixed_y(p->mp, p->g, X, Y, tw, p->stream, false); }));
+                return BORIS_OK;
+            }
+        }
         CUDA_TRY(timed(p, 1, [&] { return launch_plane_conv<T>(p->mp, (C*)p->X, (const C*)p->K, p->stream); }));
         return BORIS_OK;
     }
@@ -781,6 +791,7 @@ int mixed_setup(boris_plan p)
     if ((rc = dev_alloc(p, &p->K, mixed_kernel_entries(m) * esz))) return rc;
     CUDA_TRY(build_mixed_spectrum(p->g, m, p->dx, p->dy, p->dz, 40.0, p->K, p->f64, p->stream, p->images));
     if ((rc = dev_alloc(p, &p->X, (size_t)p->g.nkx * 3 * p->g.nz * p->g.ny * esz))) return rc;
+    if (m.split && (rc = dev_alloc(p, &p->Y, (size_t)p->g.nkx * 3 * p->g.nz * p->g.py * esz))) return rc;
     CUDA_TRY(cudaStreamSynchronize(p->stream));
     return BORIS_OK;
 }
@@ -977,15 +988,17 @@ static int plan_create(int nx, int ny, int nz, double dx, double dy, double dz, 
     p->noalloc_need = (((size_t)g.nkx * 3 * nz * ny * sizeof(float2) + 255) & ~(size_t)255) +
                       (split_fits ? (size_t)g.nkx * g.py * 3 * nz * sizeof(float2) : 0);
     // Mixed-radix lengths with the whole kx plane in one CTA's shared memory,
-    // where they pay (mixed_pays) and no switch pins another schedule;
-    // BORIS_YZ_KIND=3 takes them wherever the plane fits.
+    // or y, z and y passes, where they pay (mixed_pays) and no switch pins another
+    // schedule; BORIS_YZ_KIND=3 and 4 take the one and the other wherever they can.
     const char* kind = std::getenv("BORIS_YZ_KIND");
-    const bool forced = kind && std::atoi(kind) == 3;
+    const int fk = kind ? std::atoi(kind) : 0;
+    const bool forced = fk == 3 || fk == 4;
     bool pinned = tc != 0 || (kind && !forced);
     for (const char* v : {"BORIS_YZ_CLUSTER", "BORIS_YZ_THREADS", "BORIS_YZ_QC", "BORIS_YZ_TMA"})
         pinned |= std::getenv(v) != nullptr;
     if (const char* sf = std::getenv("BORIS_FUSE_STAGE")) pinned |= std::atoi(sf) == 1;
-    if (!pinned && mixed_plan_shape(nx, ny, nz, p->f64, max_smem, &p->mp) && (forced || mixed_pays(p->mp, p->f64, g))) {
+    if (!pinned && mixed_plan_shape(nx, ny, nz, p->f64, max_smem, fk, &p->mp) && (forced || mixed_pays(p->mp, p->f64, g)) &&
+        (!p->mp.split || split_fits)) {  // (noalloc_need has no second workspace otherwise)
         p->mixed = true;
         Geometry& mg = p->g;
         mg.px = 2 * p->mp.x.H;
@@ -999,13 +1012,12 @@ static int plan_create(int nx, int ny, int nz, double dx, double dy, double dz, 
         // their 16- and 8-row tiles (512 x 512 x 1: 5.2 against 7.1 us a pass, 512 x 512
         // x 8: 20 against 29; 1024 x 1024 x 2: 29 against 33)
         p->mixed_x1024 = !p->f64 && (mg.px == 1024 || mg.px == 2048) && (long)ny * nz >= 256;
-        if (p->mixed_x1024) {
-            mg.lgx = ilog2(mg.px);
-            mg.lmax = mg.px;
-            mg.lglmax = mg.lgx;
+        if (p->mixed_x1024 || (p->mp.split && mg.py == 1024)) {
+            mg.lmax = p->mixed_x1024 ? mg.px : 1024;
+            mg.lgx = mg.lglmax = ilog2(mg.lmax);
             if ((rc = upload_plan_twiddles(p, mg, false))) return bail(rc);
         }
-        p->yz = YZSchedule{3, 1, 0, p->mp.threads, p->mp.smem};
+        p->yz = p->mp.split ? YZSchedule{4, 1, 0, 128, 0} : YZSchedule{3, 1, 0, p->mp.threads, p->mp.smem};
         if ((rc = mixed_setup(p))) return bail(rc);
         *out = p;
         return BORIS_OK;

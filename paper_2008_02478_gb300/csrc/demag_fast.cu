@@ -12,6 +12,8 @@
 #include "boris_internal.cuh"
 #include "bulk_async.cuh"
 #include "ml_mixed.cuh"
+
+#include <type_traits>
 #include "warp_fft.cuh"
 
 namespace boris {
@@ -724,17 +726,21 @@ cudaError_t launch_ml_y_1024(const Geometry& g, const MLPlane* planes, float2* X
 {
     const size_t smem = smem_1024<float>();
     const dim3 grid((3 * g.nz + 7) / 8, g.nkx);
-    cudaError_t e;
-    if (forward) {
-        e = cudaFuncSetAttribute(y_fwd_1024_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        y_fwd_1024_kernel<float, true><<<grid, 256, smem, st>>>(g, X, Y, tw, planes);
-    } else {
-        e = cudaFuncSetAttribute(y_inv_1024_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        y_inv_1024_kernel<float, true><<<grid, 256, smem, st>>>(g, Y, X, tw, planes);
-    }
-    return cudaGetLastError();
+    auto run = [&](auto win) {
+        constexpr bool WIN = decltype(win)::value;
+        cudaError_t e;
+        if (forward) {
+            e = cudaFuncSetAttribute(y_fwd_1024_kernel<float, WIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            y_fwd_1024_kernel<float, WIN><<<grid, 256, smem, st>>>(g, X, Y, tw, planes);
+        } else {
+            e = cudaFuncSetAttribute(y_inv_1024_kernel<float, WIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            y_inv_1024_kernel<float, WIN><<<grid, 256, smem, st>>>(g, Y, X, tw, planes);
+        }
+        return cudaGetLastError();
+    };
+    return planes ? run(std::true_type{}) : run(std::false_type{});
 }
 
 // The persistent 16-bit y passes apply to even ny and 16-byte aligned arrays;

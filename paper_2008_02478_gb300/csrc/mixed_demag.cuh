@@ -15,6 +15,7 @@ struct MixedPlan {
     int nkz;          // kernel rows kz' per kx: HZ + 1, or 1
     int kyp;          // ky' entries per kernel row, H_y + 1 rounded up to 16
     size_t smem;      // shared bytes of the plane kernel
+    bool split;       // y, z and y passes over the padded spectrum instead of it (FP32)
     int threads;
     const void* twx;  // twiddle tables of the axes, in the plan's precision
     const void* twy;
@@ -45,7 +46,8 @@ constexpr int plane_h_max(size_t real_size, int cls)
 constexpr int ZTAB = 256;
 
 // Whether the mesh runs on this path (host rule); fills the axis plans.
-bool mixed_plan_shape(int nx, int ny, int nz, bool f64, int max_smem, MixedPlan* m);
+// kind 3 or 4: the plane kernel or the passes wherever possible, 0: the faster one
+bool mixed_plan_shape(int nx, int ny, int nz, bool f64, int max_smem, int kind, MixedPlan* m);
 // Whether it is the faster path there (pow2: the power-of-two geometry of the same mesh).
 bool mixed_pays(const MixedPlan& m, bool f64, const Geometry& pow2);
 // Host tables of the plan, concatenated: [twx | twy | twz], positions [posx | posy]
@@ -62,6 +64,11 @@ template <typename T>
 cudaError_t launch_mixed_x_inv(const MixedPlan& m, const typename Cx<T>::t* X, T* H, cudaStream_t st);
 template <typename T>
 cudaError_t launch_plane_conv(const MixedPlan& m, typename Cx<T>::t* X, const typename Cx<T>::t* K, cudaStream_t st);
+
+// The passes (mixed_split.cu); g, tw: the geometry and twiddles of the 1024-point kernels
+cudaError_t launch_mixed_y(const MixedPlan& m, const Geometry& g, float2* X, float2* Y, const float2* tw, cudaStream_t st,
+                           bool forward);
+cudaError_t launch_mixed_z(const MixedPlan& m, float2* Y, const float2* K, cudaStream_t st);
 
 // per-type, per-class pieces (one translation unit each)
 template <typename T> cudaError_t x_set_attr(const MixedPlan& m);

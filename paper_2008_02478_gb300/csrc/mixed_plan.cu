@@ -1,5 +1,5 @@
 // Host planning of the mixed-radix path (mixed_fft.cuh, mixed_x.cuh, plane_conv.cuh).
-#include "mixed_demag.cuh"
+#include "ml_mixed.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -72,7 +72,32 @@ void line_pos_host(const LineFFT& f, int esz, unsigned short* out)
     }
 }
 
-bool mixed_plan_shape(int nx, int ny, int nz, bool f64, int max_smem, MixedPlan* m)
+// Times of the y-z part, us, fitted to measurements of FP32 meshes.
+//
+// One CTA carries a whole plane: the points of the planes an SM gets, 0.95e-3
+// each with two or more CTAs per SM (256 x 256 x 8: 23.6 us), 1.1e-3 with one and
+// HZ <= 8 (512 x 512 x 8: 105), 1.45e-3 to HZ 24 (160 x 160 x 20: 53), 1.75e-3 beyond
+// (128 x 128 x 32: 43), and 15 % more with radices 20 and 24 (480 x 480 x 8: 116).
+static double plane_us(const MixedPlan& m)
+{
+    const double w = 3.0 * m.nz * 2.0 * m.y.H;
+    const int planes = m.x.H + 1, res = (int)(228 * 1024 / (m.smem + 1024)), per_sm = (planes + 151) / 152;
+    const double one = m.HZ <= 8 ? 1.1e-3 : m.HZ <= 24 ? 1.6e-3 : 1.75e-3;
+    const double many = res >= 2 ? 0.95e-3 : m.HZ <= 8 ? 1.1e-3 : m.HZ <= 24 ? 1.45e-3 : 1.75e-3;
+    return (m.y.H == 480 && m.cls > 0 ? 1.15 : 1.0) * std::max(one * w, per_sm * w * many);
+}
+// y passes 7e-6 per point (160 x 640 x 12: 57 us), 8e-6 with radix 20 and 10e-6 from
+// 1536 points (545 x 836 x 6: 213), 4.8e-6 with 1024; z pass 5e-6 to HZ 8 (107), 8e-6
+// to 16 (160 x 640 x 12: 59), 6.5e-6 with 20 (160 x 160 x 20: 25), 10.5e-6 with 24 (283 x 269
+// x 24: 152), 18e-6 with 32.
+static double passes_us(const MixedPlan& m)
+{
+    const double y = m.y.H == 512 ? 4.8e-6 : m.y.H >= 768 ? 10e-6 : m.y.H % 240 == 0 ? 8e-6 : 7e-6;
+    const double z = m.HZ <= 8 ? 5e-6 : m.HZ <= 16 ? 8e-6 : m.HZ <= 20 ? 6.5e-6 : m.HZ <= 24 ? 10.5e-6 : 18e-6;
+    return (m.HZ <= 24 ? 9.0 : 16.0) + (m.x.H + 1) * 3.0 * m.nz * 2.0 * m.y.H * (y + z);
+}
+
+bool mixed_plan_shape(int nx, int ny, int nz, bool f64, int max_smem, int kind, MixedPlan* m)
 {
     const int csz = f64 ? 16 : 8;
     if (nx < 2 || ny < 2 || nz < 1) return false;
@@ -105,8 +130,26 @@ bool mixed_plan_shape(int nx, int ny, int nz, bool f64, int max_smem, MixedPlan*
     if (m->cls > 0) make_line_fft(ny, csz, true, &m->y);
     m->kyp = (m->y.H + 1 + 15) / 16 * 16;
     m->smem = (size_t)3 * nz * m->y.LS * csz;
-    if (m->smem > (size_t)max_smem || m->y.H > plane_h_max(rs, m->cls)) return false;
     if ((size_t)2 * m->x.LS * csz > (size_t)max_smem) return false;
+    const bool fits = m->smem <= (size_t)max_smem && m->y.H <= plane_h_max(rs, m->cls);
+    if (!f64 && nz > 1 && kind != 3) {
+        MixedPlan s = *m;
+        s.split = true;
+        if (s.cls == 0) s.cls = 1;
+        make_line_fft(ny, csz, true, &s.y);
+        s.kyp = (s.y.H + 1 + 15) / 16 * 16;
+        s.smem = 0;
+        s.threads = 128;
+        // few planes of many points leave most SMs idle (36 x 229 x 13, 41 planes: 29 us an
+        // evaluation against 40), and 161 planes make two rounds of 152 SMs (160 x 160 x 20:
+        // 63 against 69)
+        if (kind == 4 || !fits || passes_us(s) < 0.98 * plane_us(*m)) {
+            *m = s;
+            return (size_t)m->y.LS * csz <= (size_t)max_smem;
+        }
+    }
+    m->split = false;
+    if (!fits || kind == 4) return false;
     // threads per CTA: the register file shared by as many CTAs as it takes to
     // hold all planes at once (up to four, and up to what shared memory allows):
     // one wave of smaller CTAs beats two of larger ones (512 x 512 x 1: 128
@@ -121,25 +164,30 @@ bool mixed_plan_shape(int nx, int ny, int nz, bool f64, int max_smem, MixedPlan*
 
 bool mixed_pays(const MixedPlan& m, bool f64, const Geometry& pow2)
 {
-    // One CTA carries a whole plane: the time is the points of the planes an SM
-    // gets, while the power-of-two schedules spread all points over the chip but
-    // have more of them.  Measured, us per point: FP32 0.95e-3 with two or more
-    // CTAs per SM (256 x 256 x 8: 23.6 us), 1.1e-3 with one and HZ <= 8 (512 x 512 x 8:
-    // 105 us), 1.45e-3 to HZ 24 (160 x 160 x 20: 53 us), 1.75e-3 beyond (128 x 128 x 32:
-    // 43 us); the split schedule 8.8e-6 over all planes plus 6 us, 16 us at least
-    // (256 x 256 x 16: 55 us against 75 here; 27 x 137 x 26, 33 planes of 25 k points: 22
-    // against 51).  FP64 is bound by its arithmetic units: 25e-3 (one plane) to 40e-3
-    // (128 x 128 x 16: 490 us) against 2.2e-4 to 3.2e-4 (564 us).
-    const double w = 3.0 * m.nz * 2.0 * m.y.H;
-    const int planes = m.x.H + 1, res = (int)(228 * 1024 / (m.smem + 1024)), per_sm = (planes + 151) / 152;
+    // The power-of-two schedules spread all points over the chip but have more of them.
     const double all = 3.0 * m.nz * pow2.py * (double)pow2.nkx;
     if (f64) {
+        // bound by the arithmetic units: 25e-3 (one plane) to 40e-3 per point (128 x 128
+        // x 16: 490 us) against 2.2e-4 to 3.2e-4 over all planes (564 us)
+        const double w = 3.0 * m.nz * 2.0 * m.y.H, per_sm = (m.x.H + 152) / 152;
         const double c = m.HZ == 1 ? 25e-3 : m.HZ <= 4 ? 31e-3 : m.HZ <= 8 ? 36e-3 : 40e-3;
         return per_sm * w * c <= std::max(15.0, all * (m.HZ == 1 ? 2.2e-4 : m.HZ <= 4 ? 2.4e-4 : 3.2e-4));
     }
-    const double one = m.HZ <= 8 ? 1.1e-3 : m.HZ <= 24 ? 1.6e-3 : 1.75e-3;
-    const double many = res >= 2 ? 0.95e-3 : m.HZ <= 8 ? 1.1e-3 : m.HZ <= 24 ? 1.45e-3 : 1.75e-3;
-    return std::max(one * w, per_sm * w * many) <= 1.15 * std::max(16.0, 6.0 + all * 8.8e-6);
+    // their x passes take longer on short rows, per row and evaluation 3.8e-3 us to
+    // 128 points (37 x 398 x 16: 35 against 11 us), 2e-3 with 256, 0.6e-3 with 512
+    const double x = (double)m.y.n * m.nz * (pow2.px <= 128 ? 3.8e-3 : pow2.px == 256 ? 2e-3 : pow2.px == 512 ? 0.6e-3 : 0.0);
+    if (m.split) {
+        // 20 us (10 with 33 planes: 27 x 137 x 26 23) plus 7.7e-6 for a full z axis (320 x 388 x 16: 200), more with padding in z
+        // (283 x 269 x 24: 370), an eighth more from 2048 points in y (160 x 640 x 12: 205);
+        // taken from 8 % less on (197 x 769 x 10, not taken: 227 against 306)
+        const double pad = 0.6 + 0.2 * pow2.pz / m.nz;
+        return passes_us(m) <= 0.92 * ((pow2.px <= 64 ? 10.0 : 20.0) + all * 7.7e-6 * pad) * (pow2.py >= 2048 ? 1.12 : 1.0) + x;
+    }
+    // 8.8e-6 plus 6 us, 16 us at least and 25 from HZ 12 and 128 x points on (256 x 256 x 16: 55 us
+    // against 75 in planes; 27 x 137 x 26, 33 planes of 25 k points: 22 against 51; 34 x 88
+    // x 22: 31 against 22); with fewer points in x, too, 15 % more
+    const double gain = 2 * m.x.H < pow2.px ? 1.15 : 0.98;
+    return plane_us(m) <= gain * std::max(m.HZ <= 8 || pow2.px <= 64 ? 16.0 : 25.0, 6.0 + all * 8.8e-6) + x;
 }
 
 size_t mixed_tw_entries(const MixedPlan& m, size_t* oy, size_t* oz)
@@ -191,7 +239,14 @@ static cudaError_t prepare_t(const MixedPlan& m)
     default: return plane_set_attr<T, 3>();
     }
 }
-cudaError_t mixed_prepare(const MixedPlan& m, bool f64) { return f64 ? prepare_t<double>(m) : prepare_t<float>(m); }
+cudaError_t mixed_prepare(const MixedPlan& m, bool f64)
+{
+    if (m.split) {
+        const cudaError_t e = x_set_attr<float>(m);
+        return e == cudaSuccess ? line_y_prepare(m) : e;
+    }
+    return f64 ? prepare_t<double>(m) : prepare_t<float>(m);
+}
 
 template <typename T>
 cudaError_t launch_plane_conv(const MixedPlan& m, typename Cx<T>::t* X, const typename Cx<T>::t* K, cudaStream_t st)

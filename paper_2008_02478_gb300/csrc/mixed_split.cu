@@ -1,0 +1,93 @@
+// The y-z part of the convolution on mixed-radix lengths as three passes over
+// the padded spectrum: y transforms X[kx][c][z][y] -> Y[kx][c][z][ky] (those of
+// ml_mixed_y.cu), the z stage in place on Y, y inverses.  For meshes whose plane
+// does not fit one CTA's shared memory, or whose planes leave SMs idle, where
+// the power-of-two lengths pad most (mixed_pays): the z stage, the transforms of
+// plane_conv.cuh, reaches a third of the copy rate (latency: 12 to 20 warps per
+// SM), the power-of-two one two thirds.  Evaluations, before -> now: 160 x 640 x 12
+// 238 -> 149 us, 86 x 705 x 8 87 -> 53, 39 x 143 x 23 56 -> 33, 283 x 269 x 24 412 -> 320,
+// 545 x 836 x 6 525 -> 436 (power-of-two passes), 160 x 160 x 20 69 -> 63 (planes).
+#include "bulk_async.cuh"
+#include "ml_mixed.cuh"
+#include "plane_conv.cuh"
+
+namespace boris {
+
+namespace {
+
+// Four warps per CTA, the items of all kx side by side (545 x 836 x 6: 126 us with
+// those of one kx side by side, now 107).  HZ 16 to 24: TK bins ky' of one kx and
+// their mirrors go through shared memory in rows of 256 consecutive bytes,
+// [line][TK | 8 | TK] (the gap keeps a bin and its mirror in different banks);
+// with other lengths each warp reads and writes one item's columns in 32- to
+// 64-byte pieces (staged against direct: 80 x 897 x 23 121 and 171 us, 128 x 200 x 20 28
+// and 35; 545 x 836 x 6 155 and 120, 300 x 400 x 8 47 and 35).
+constexpr int TK = 32, ZLS = 2 * TK + 8;
+constexpr bool z_staged(int HZ) { return HZ >= 16 && HZ <= 24; }
+
+template <int HZ, int RES>
+__global__ void __launch_bounds__(128, z_staged(HZ) ? 3 : HZ <= 12 ? 5 : 2) z_conv_kernel(int H, int nz, int kyp, int nkz, float2* __restrict__ Y,
+                                                     const float2* __restrict__ K, const float2* __restrict__ twz)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int KB = 16 / RES;
+    const int P = 2 * H, kx = blockIdx.x, k0 = blockIdx.y * TK;
+    float2* base = Y + (size_t)kx * 3 * nz * P;
+    const float2* Kx = K + (size_t)kx * nkz * 3 * kyp;
+    const int warp = threadIdx.x >> 5, items = H / KB + 1;
+    if constexpr (z_staged(HZ)) {
+        float2* buf = reinterpret_cast<float2*>(smem_raw);
+        const int half = (threadIdx.x >> 5) & 1, col = threadIdx.x & 31, k = k0 + col;
+        const bool ok = half ? k > 0 && k < H : k <= H;
+        const int ky = ok ? (half ? P - k : k) : 0, at = col + half * (TK + 8);
+        for (int l = threadIdx.x >> 6; l < 3 * nz; l += 2)
+            if (ok)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(buf + l * ZLS + at)),
+                             "l"(base + (size_t)l * P + ky)
+                             : "memory");
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+        z_columns<float, HZ, RES>(H, ZLS, nz * ZLS, nz, kyp, Kx, twz, k0 / KB + warp, min(k0 / KB + TK / KB, items), 4,
+                                  [&](int q) { return buf + (q <= H ? q - k0 : P - q - k0 + TK + 8); });
+        __syncthreads();
+        if (ok)
+            for (int l = threadIdx.x >> 6; l < 3 * nz; l += 2) base[(size_t)l * P + ky] = buf[l * ZLS + at];
+    } else {
+        // one item per warp
+        z_columns<float, HZ, RES>(H, P, nz * P, nz, kyp, Kx, twz, blockIdx.y * 4 + warp, items, items, [&](int q) { return base + q; });
+    }
+}
+
+template <int HZ>
+cudaError_t z_launch(const MixedPlan& m, float2* Y, const float2* K, cudaStream_t st)
+{
+    constexpr int RES = HZ <= 8 ? 2 : 4;
+    const size_t smem = z_staged(HZ) ? (size_t)3 * m.nz * ZLS * sizeof(float2) : 0;  // 41 KB at most
+    const int tiles = z_staged(HZ) ? m.y.H / TK + 1 : (m.y.H * RES / 16 + 4) / 4;
+    z_conv_kernel<HZ, RES><<<dim3(m.x.H + 1, tiles), 128, smem, st>>>(m.y.H, m.nz, m.kyp, m.nkz, Y, K,
+                                                                             (const float2*)m.twz);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_mixed_z(const MixedPlan& m, float2* Y, const float2* K, cudaStream_t st)
+{
+    switch (m.HZ) {
+#define Z(h) \
+    case h: return z_launch<h>(m, Y, K, st);
+        Z(2) Z(4) Z(6) Z(8) Z(12) Z(16) Z(20) Z(24) Z(32)
+#undef Z
+    }
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_mixed_y(const MixedPlan& m, const Geometry& g, float2* X, float2* Y, const float2* tw, cudaStream_t st,
+                           bool forward)
+{
+    // 1024 points: the warp-held transforms (one trip through shared memory)
+    if (m.y.H == 512) return launch_ml_y_1024(g, nullptr, X, Y, tw, st, forward);
+    return launch_line_y(m, nullptr, 3 * m.nz, m.nz, X, Y, st, forward);
+}
+
+}  // namespace boris

@@ -144,7 +144,7 @@ cudaError_t ml_mixed_prepare(const MLMixed& p)
         if (r != cudaSuccess) return r;
         return cudaFuncSetAttribute(ml_x_inv_kernel<decltype(L)>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     });
-    return e == cudaSuccess ? ml_y_prepare(p) : e;
+    return e == cudaSuccess ? line_y_prepare(p.m) : e;
 }
 
 cudaError_t launch_ml_x_fwd(const MLMixed& p, const float* M, const float* ms_map, float ms, float2* X, cudaStream_t st)

@@ -100,7 +100,13 @@ extern "C" int boris_demag_apply_noalloc(boris_plan p, const float* M, float* Hd
     if (v.mixed) {
         e = v.mixed_x1024 ? launch_x_r2c<float>(v.g, M, nullptr, 1.0f, X, tw, v.stream)
                           : launch_mixed_x_fwd<float>(*v.mixed, M, nullptr, 1.0f, X, v.stream);
-        if (e == cudaSuccess) e = launch_plane_conv<float>(*v.mixed, X, (const float2*)v.K, v.stream);
+        if (e == cudaSuccess && v.mixed->split) {
+            e = launch_mixed_y(*v.mixed, v.g, X, Y, tw, v.stream, true);
+            if (e == cudaSuccess) e = launch_mixed_z(*v.mixed, Y, (const float2*)v.K, v.stream);
+            if (e == cudaSuccess) e = launch_mixed_y(*v.mixed, v.g, X, Y, tw, v.stream, false);
+        } else if (e == cudaSuccess) {
+            e = launch_plane_conv<float>(*v.mixed, X, (const float2*)v.K, v.stream);
+        }
         if (e == cudaSuccess)
             e = v.mixed_x1024 ? launch_x_c2r<float>(v.g, X, Hd, tw, v.stream)
                               : launch_mixed_x_inv<float>(*v.mixed, X, Hd, v.stream);

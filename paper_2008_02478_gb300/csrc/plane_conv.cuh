@@ -94,6 +94,98 @@ __device__ __noinline__ void y_inverse(typename Cx<T>::t* __restrict__ plane, in
     });
 }
 
+// The z transforms, kernel multiply and inverses of the columns ky' = KB w .. of
+// items w = w0, w0 + wstep, ... < wend: column(ky) is row 0 of component 0, rows LS and
+// components cs apart.
+template <typename T, int HZ, int RES, typename Col>
+__device__ __forceinline__ void z_columns(int H, int LS, int cs, int nz, int kyp, const typename Cx<T>::t* __restrict__ Kx,
+                                          const typename Cx<T>::t* __restrict__ twz, int w0, int wend, int wstep, Col column)
+{
+    using C = typename Cx<T>::t;
+    constexpr int Q = RES == 2 ? HZ : HZ / 2;  // points of a lane's DFT
+    constexpr int HQ = Q / 2;
+    constexpr int KB = 16 / RES;  // ky' per warp item
+    static_assert(Q % 2 == 0, "the halving exchange needs an even number of points");
+    const int lane = threadIdx.x & 31;
+    const int res = lane & (RES - 1), kl = (lane & 15) / RES;
+    const bool mirror = lane & 16, odd = lane & 1, up = RES == 4 && (lane & 2);
+    const T sy = mirror ? T(-1) : T(1), so = odd ? T(-1) : T(1), syo = sy * so;
+    const C* tz = twz + res * 4 * Q;  // rows: in (x[m]), in (x[m + Q]), keep, send
+    const int krow = 3 * kyp;
+    for (int w = w0; w < wend; w += wstep) {  // (the same for all lanes of a warp)
+        const int k = w * KB + kl;
+        const bool ok = k <= H && !(mirror && (k == 0 || k == H));
+        const int kc = k <= H ? k : H;  // in range for the loads of idle lanes
+        C* col = column(mirror ? (kc == 0 ? 0 : 2 * H - kc) : kc);
+        C u[3][Q];
+#pragma unroll
+        for (int m = 0; m < Q; m++) {
+            const C wa = __ldg(tz + m);
+#pragma unroll
+            for (int c = 0; c < 3; c++)
+                u[c][m] = m < nz ? c_mul(col[c * cs + m * LS], wa) : C{T(0), T(0)};
+            if (RES == 4) {
+                const C wb = __ldg(tz + Q + m);
+                if (m + Q < nz) {
+#pragma unroll
+                    for (int c = 0; c < 3; c++) {
+                        const C x = col[c * cs + (m + Q) * LS];
+                        u[c][m].x += x.x * wb.x - x.y * wb.y;
+                        u[c][m].y += x.x * wb.y + x.y * wb.x;
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 3; c++) dft<Q, -1>(u[c]);
+        // kz = RES j + r; rows past kz = HZ are the mirror image kz' = 2 HZ - kz
+        // (odd entries negated; at kz = HZ they are zero, so its sign does not matter)
+        const C* Ku = Kx + kc + res * krow;
+        const C* Kd = Kx + kc + (2 * HZ - res) * krow;
+#pragma unroll
+        for (int j = 0; j < Q; j++) {
+            const bool fz = j >= Q / 2;
+            const C* kp = fz ? Kd - RES * j * krow : Ku + RES * j * krow;
+            const C d01 = __ldg(kp), d23 = __ldg(kp + kyp), d45 = __ldg(kp + 2 * kyp);
+            const T s = j & 1 ? so : T(1), t = j & 1 ? syo : sy;
+            constexpr auto pm = &Radix<Q>::perm;
+            kernel_mult<T>(d01, d23, d45, s, t, fz ? -s : s, fz ? -t : t, u[0][pm(j)], u[1][pm(j)], u[2][pm(j)]);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; c++) dft<Q, 1>(u[c]);
+#pragma unroll
+        for (int m = 0; m < Q; m++) {
+            const C wk = __ldg(tz + 2 * Q + m);
+            if (RES == 4) {
+                const C ws = __ldg(tz + 3 * Q + m);
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    const C got = shfl_x(c_mul(u[c][m], ws), 2);
+                    u[c][m] = c_add(c_mul(u[c][m], wk), got);
+                }
+            } else {
+#pragma unroll
+                for (int c = 0; c < 3; c++) u[c][m] = c_mul(u[c][m], wk);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < 3; c++)
+#pragma unroll
+            for (int m = 0; m < HQ; m++) u[c][m] = c_add(u[c][m], shfl_x(u[c][m + HQ], 1));
+        __syncwarp();
+        const int row0 = (odd ? HQ : 0) + (up ? Q : 0);
+        if (ok) {
+#pragma unroll
+            for (int m = 0; m < HQ; m++) {
+                if (row0 + m < nz) {
+#pragma unroll
+                    for (int c = 0; c < 3; c++) col[c * cs + (row0 + m) * LS] = u[c][m];
+                }
+            }
+        }
+    }
+}
+
 template <typename T, int HZ, int RES>
 __device__ __noinline__ void z_stage(int H, int LS, int nz, int kyp, const typename Cx<T>::t* __restrict__ Kx,
                                      const typename Cx<T>::t* __restrict__ twz, const unsigned short* __restrict__ pos)
@@ -113,90 +205,9 @@ __device__ __noinline__ void z_stage(int H, int LS, int nz, int kyp, const typen
             }
         }
     } else {
-        constexpr int Q = RES == 2 ? HZ : HZ / 2;  // points of a lane's DFT
-        constexpr int HQ = Q / 2;
-        constexpr int KB = 16 / RES;  // ky' per warp item
-        static_assert(Q % 2 == 0, "the halving exchange needs an even number of points");
-        const int lane = threadIdx.x & 31;
-        const int res = lane & (RES - 1), kl = (lane & 15) / RES;
-        const bool mirror = lane & 16, odd = lane & 1, up = RES == 4 && (lane & 2);
-        const T sy = mirror ? T(-1) : T(1), so = odd ? T(-1) : T(1), syo = sy * so;
-        const int cs = nz * LS;  // component stride
-        const C* tz = twz + res * 4 * Q;  // rows: in (x[m]), in (x[m + Q]), keep, send
-        const int krow = 3 * kyp;
         // blockDim is a multiple of 32: a warp's lanes leave the loop together
-        for (int w = threadIdx.x >> 5; w * KB <= H; w += blockDim.x >> 5) {
-            const int k = w * KB + kl;
-            const bool ok = k <= H && !(mirror && (k == 0 || k == H));
-            const int kc = k <= H ? k : H;  // in range for the loads of idle lanes
-            C* col = buf + pos[mirror ? (kc == 0 ? 0 : 2 * H - kc) : kc];
-            C u[3][Q];
-#pragma unroll
-            for (int m = 0; m < Q; m++) {
-                const C wa = __ldg(tz + m);
-#pragma unroll
-                for (int c = 0; c < 3; c++)
-                    u[c][m] = m < nz ? c_mul(col[c * cs + m * LS], wa) : C{T(0), T(0)};
-                if (RES == 4) {
-                    const C wb = __ldg(tz + Q + m);
-                    if (m + Q < nz) {
-#pragma unroll
-                        for (int c = 0; c < 3; c++) {
-                            const C x = col[c * cs + (m + Q) * LS];
-                            u[c][m].x += x.x * wb.x - x.y * wb.y;
-                            u[c][m].y += x.x * wb.y + x.y * wb.x;
-                        }
-                    }
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < 3; c++) dft<Q, -1>(u[c]);
-            // kz = RES j + r; rows past kz = HZ are the mirror image kz' = 2 HZ - kz
-            // (odd entries negated; at kz = HZ they are zero, so its sign does not matter)
-            const C* Ku = Kx + kc + res * krow;
-            const C* Kd = Kx + kc + (2 * HZ - res) * krow;
-#pragma unroll
-            for (int j = 0; j < Q; j++) {
-                const bool fz = j >= Q / 2;
-                const C* kp = fz ? Kd - RES * j * krow : Ku + RES * j * krow;
-                const C d01 = __ldg(kp), d23 = __ldg(kp + kyp), d45 = __ldg(kp + 2 * kyp);
-                const T s = j & 1 ? so : T(1), t = j & 1 ? syo : sy;
-                constexpr auto pm = &Radix<Q>::perm;
-                kernel_mult<T>(d01, d23, d45, s, t, fz ? -s : s, fz ? -t : t, u[0][pm(j)], u[1][pm(j)], u[2][pm(j)]);
-            }
-#pragma unroll
-            for (int c = 0; c < 3; c++) dft<Q, 1>(u[c]);
-#pragma unroll
-            for (int m = 0; m < Q; m++) {
-                const C wk = __ldg(tz + 2 * Q + m);
-                if (RES == 4) {
-                    const C ws = __ldg(tz + 3 * Q + m);
-#pragma unroll
-                    for (int c = 0; c < 3; c++) {
-                        const C got = shfl_x(c_mul(u[c][m], ws), 2);
-                        u[c][m] = c_add(c_mul(u[c][m], wk), got);
-                    }
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 3; c++) u[c][m] = c_mul(u[c][m], wk);
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < 3; c++)
-#pragma unroll
-                for (int m = 0; m < HQ; m++) u[c][m] = c_add(u[c][m], shfl_x(u[c][m + HQ], 1));
-            __syncwarp();
-            const int row0 = (odd ? HQ : 0) + (up ? Q : 0);
-            if (ok) {
-#pragma unroll
-                for (int m = 0; m < HQ; m++) {
-                    if (row0 + m < nz) {
-#pragma unroll
-                        for (int c = 0; c < 3; c++) col[c * cs + (row0 + m) * LS] = u[c][m];
-                    }
-                }
-            }
-        }
+        z_columns<T, HZ, RES>(H, LS, nz * LS, nz, kyp, Kx, twz, threadIdx.x >> 5, H * RES / 16 + 1, blockDim.x >> 5,
+                              [&](int ky) { return buf + pos[ky]; });
     }
     __syncthreads();
 }
