@@ -93,8 +93,8 @@ def test_persistent_sum_over_plane_counts(planes, ny, variant, monkeypatch):
     sources below, above and between a warp's targets; one and several column
     tiles.  Sampled cells of the direct sum."""
     torch = torch_cuda()
-    if variant == 3 and sum(planes) > 36:
-        pytest.skip("two blocks per SM hold 36 planes")
+    if variant == 3 and sum(planes) > 35:
+        pytest.skip("two blocks per SM hold 35 planes")
     monkeypatch.setenv("BORIS_ML_MIX", str(variant))
     st, m, M, plan = make_case([(5 - l, ny - l, nz) for l, nz in enumerate(planes)])
     assert plan.schedule()[2] == variant
