@@ -88,12 +88,12 @@ static double plane_us(const MixedPlan& m)
 }
 // y passes 7e-6 per point (160 x 640 x 12: 57 us), 8e-6 with radix 20 and 10e-6 from
 // 1536 points (545 x 836 x 6: 213), 4.8e-6 with 1024; z pass 5e-6 to HZ 8 (107), 8e-6
-// to 16 (160 x 640 x 12: 59), 6.5e-6 with 20 (160 x 160 x 20: 25), 10.5e-6 with 24 (283 x 269
-// x 24: 152), 18e-6 with 32.
+// to 16 (160 x 640 x 12: 59), 6.5e-6 with 20 (160 x 160 x 20: 23), 8.3e-6 with 24 (283 x 269
+// x 24: 122), 18e-6 with 32.
 static double passes_us(const MixedPlan& m)
 {
     const double y = m.y.H == 512 ? 4.8e-6 : m.y.H >= 768 ? 10e-6 : m.y.H % 240 == 0 ? 8e-6 : 7e-6;
-    const double z = m.HZ <= 8 ? 5e-6 : m.HZ <= 16 ? 8e-6 : m.HZ <= 20 ? 6.5e-6 : m.HZ <= 24 ? 10.5e-6 : 18e-6;
+    const double z = m.HZ <= 8 ? 5e-6 : m.HZ <= 16 ? 8e-6 : m.HZ <= 20 ? 6.5e-6 : m.HZ <= 24 ? 8.3e-6 : 18e-6;
     return (m.HZ <= 24 ? 9.0 : 16.0) + (m.x.H + 1) * 3.0 * m.nz * 2.0 * m.y.H * (y + z);
 }
 
@@ -142,7 +142,7 @@ bool mixed_plan_shape(int nx, int ny, int nz, bool f64, int max_smem, int kind, 
         s.threads = 128;
         // few planes of many points leave most SMs idle (36 x 229 x 13, 41 planes: 29 us an
         // evaluation against 40), and 161 planes make two rounds of 152 SMs (160 x 160 x 20:
-        // 63 against 69)
+        // 62 against 69)
         if (kind == 4 || !fits || passes_us(s) < 0.98 * plane_us(*m)) {
             *m = s;
             return (size_t)m->y.LS * csz <= (size_t)max_smem;

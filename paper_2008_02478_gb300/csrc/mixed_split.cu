@@ -3,10 +3,10 @@
 // ml_mixed_y.cu), the z stage in place on Y, y inverses.  For meshes whose plane
 // does not fit one CTA's shared memory, or whose planes leave SMs idle, where
 // the power-of-two lengths pad most (mixed_pays): the z stage, the transforms of
-// plane_conv.cuh, reaches a third of the copy rate (latency: 12 to 20 warps per
-// SM), the power-of-two one two thirds.  Evaluations, before -> now: 160 x 640 x 12
-// 238 -> 149 us, 86 x 705 x 8 87 -> 53, 39 x 143 x 23 56 -> 33, 283 x 269 x 24 412 -> 320,
-// 545 x 836 x 6 525 -> 436 (power-of-two passes), 160 x 160 x 20 69 -> 63 (planes).
+// plane_conv.cuh, reaches a third of the copy rate (loads' latency at 12 to 20
+// warps per SM), the power-of-two one two thirds.  Evaluations, before -> now: 160 x 640 x 12
+// 238 -> 149 us, 86 x 705 x 8 87 -> 53, 39 x 143 x 23 56 -> 32, 283 x 269 x 24 412 -> 290,
+// 545 x 836 x 6 525 -> 436 (power-of-two passes), 160 x 160 x 20 69 -> 62 (planes).
 #include "bulk_async.cuh"
 #include "ml_mixed.cuh"
 #include "plane_conv.cuh"
@@ -21,8 +21,11 @@ namespace {
 // [line][TK | 8 | TK] (the gap keeps a bin and its mirror in different banks);
 // with other lengths each warp reads and writes one item's columns in 32- to
 // 64-byte pieces (staged against direct: 80 x 897 x 23 121 and 171 us, 128 x 200 x 20 28
-// and 35; 545 x 836 x 6 155 and 120, 300 x 400 x 8 47 and 35).
+// and 35; 545 x 836 x 6 155 and 120, 300 x 400 x 8 47 and 35).  The kernel rows of the
+// tile come with the columns: read where they are used, they were what the
+// warps waited for (283 x 269 x 24: 153 us, now 122; 80 x 897 x 23 115, now 90).
 constexpr int TK = 32, ZLS = 2 * TK + 8;
+constexpr int KP = 44;  // pitch of a staged kernel row: the rows of four residues start four pairs apart mod 16
 constexpr bool z_staged(int HZ) { return HZ >= 16 && HZ <= 24; }
 
 template <int HZ, int RES>
@@ -45,9 +48,14 @@ __global__ void __launch_bounds__(128, z_staged(HZ) ? 3 : HZ <= 12 ? 5 : 2) z_co
                 asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(buf + l * ZLS + at)),
                              "l"(base + (size_t)l * P + ky)
                              : "memory");
+        float2* kbuf = buf + 3 * nz * ZLS;  // [kz'][pair][KP]
+        for (int i = threadIdx.x; i < nkz * 3 * (TK / 2); i += 128) {
+            const int r = i / (TK / 2), pc = 2 * (i % (TK / 2));
+            if (k0 + pc < kyp) cp_async16(kbuf + r * KP + pc, Kx + (size_t)r * kyp + k0 + pc);
+        }
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
-        z_columns<float, HZ, RES>(H, ZLS, nz * ZLS, nz, kyp, Kx, twz, k0 / KB + warp, min(k0 / KB + TK / KB, items), 4,
+        z_columns<float, HZ, RES, true>(H, ZLS, nz * ZLS, nz, KP, kbuf - k0, twz, k0 / KB + warp, min(k0 / KB + TK / KB, items), 4,
                                   [&](int q) { return buf + (q <= H ? q - k0 : P - q - k0 + TK + 8); });
         __syncthreads();
         if (ok)
@@ -62,7 +70,9 @@ template <int HZ>
 cudaError_t z_launch(const MixedPlan& m, float2* Y, const float2* K, cudaStream_t st)
 {
     constexpr int RES = HZ <= 8 ? 2 : 4;
-    const size_t smem = z_staged(HZ) ? (size_t)3 * m.nz * ZLS * sizeof(float2) : 0;  // 41 KB at most
+    const size_t smem = z_staged(HZ) ? ((size_t)3 * m.nz * ZLS + (size_t)3 * m.nkz * KP) * sizeof(float2) : 0;  // 68 KB at most
+    const cudaError_t e = cudaFuncSetAttribute(z_conv_kernel<HZ, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
     const int tiles = z_staged(HZ) ? m.y.H / TK + 1 : (m.y.H * RES / 16 + 4) / 4;
     z_conv_kernel<HZ, RES><<<dim3(m.x.H + 1, tiles), 128, smem, st>>>(m.y.H, m.nz, m.kyp, m.nkz, Y, K,
                                                                              (const float2*)m.twz);

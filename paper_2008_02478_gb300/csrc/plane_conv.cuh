@@ -96,8 +96,8 @@ __device__ __noinline__ void y_inverse(typename Cx<T>::t* __restrict__ plane, in
 
 // The z transforms, kernel multiply and inverses of the columns ky' = KB w .. of
 // items w = w0, w0 + wstep, ... < wend: column(ky) is row 0 of component 0, rows LS and
-// components cs apart.
-template <typename T, int HZ, int RES, typename Col>
+// components cs apart.  KSH: the kernel rows (pitch kyp) are in shared memory.
+template <typename T, int HZ, int RES, bool KSH = false, typename Col>
 __device__ __forceinline__ void z_columns(int H, int LS, int cs, int nz, int kyp, const typename Cx<T>::t* __restrict__ Kx,
                                           const typename Cx<T>::t* __restrict__ twz, int w0, int wend, int wstep, Col column)
 {
@@ -146,7 +146,7 @@ __device__ __forceinline__ void z_columns(int H, int LS, int cs, int nz, int kyp
         for (int j = 0; j < Q; j++) {
             const bool fz = j >= Q / 2;
             const C* kp = fz ? Kd - RES * j * krow : Ku + RES * j * krow;
-            const C d01 = __ldg(kp), d23 = __ldg(kp + kyp), d45 = __ldg(kp + 2 * kyp);
+            const C d01 = KSH ? kp[0] : __ldg(kp), d23 = KSH ? kp[kyp] : __ldg(kp + kyp), d45 = KSH ? kp[2 * kyp] : __ldg(kp + 2 * kyp);
             const T s = j & 1 ? so : T(1), t = j & 1 ? syo : sy;
             constexpr auto pm = &Radix<Q>::perm;
             kernel_mult<T>(d01, d23, d45, s, t, fz ? -s : s, fz ? -t : t, u[0][pm(j)], u[1][pm(j)], u[2][pm(j)]);
