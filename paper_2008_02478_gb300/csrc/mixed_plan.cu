@@ -87,14 +87,14 @@ static double plane_us(const MixedPlan& m)
     return (m.y.H == 480 && m.cls > 0 ? 1.15 : 1.0) * std::max(one * w, per_sm * w * many);
 }
 // y passes 7e-6 per point (160 x 640 x 12: 57 us), 8e-6 with radix 20 and 10e-6 from
-// 1536 points (545 x 836 x 6: 213), 4.8e-6 with 1024; z pass 5e-6 to HZ 8 (107), 8e-6
-// to 16 (160 x 640 x 12: 59), 6.5e-6 with 20 (160 x 160 x 20: 23), 8.3e-6 with 24 (283 x 269
-// x 24: 122), 18e-6 with 32.
+// 1536 points (545 x 836 x 6: 213), 4.8e-6 with 1024; z pass 5e-6 to HZ 8 (107), 5.8e-6
+// with 12 (160 x 640 x 12: 42), 8e-6 with 16, 6.5e-6 with 20 (160 x 160 x 20: 23), 8.3e-6
+// with 24 (283 x 269 x 24: 122), 9.5e-6 with 32 (55 x 767 x 26: 80).
 static double passes_us(const MixedPlan& m)
 {
     const double y = m.y.H == 512 ? 4.8e-6 : m.y.H >= 768 ? 10e-6 : m.y.H % 240 == 0 ? 8e-6 : 7e-6;
-    const double z = m.HZ <= 8 ? 5e-6 : m.HZ <= 16 ? 8e-6 : m.HZ <= 20 ? 6.5e-6 : m.HZ <= 24 ? 8.3e-6 : 18e-6;
-    return (m.HZ <= 24 ? 9.0 : 16.0) + (m.x.H + 1) * 3.0 * m.nz * 2.0 * m.y.H * (y + z);
+    const double z = m.HZ <= 8 ? 5e-6 : m.HZ <= 12 ? 5.8e-6 : m.HZ <= 16 ? 8e-6 : m.HZ <= 20 ? 6.5e-6 : m.HZ <= 24 ? 8.3e-6 : 9.5e-6;
+    return (m.HZ <= 24 ? 9.0 : 12.0) + (m.x.H + 1) * 3.0 * m.nz * 2.0 * m.y.H * (y + z);
 }
 
 bool mixed_plan_shape(int nx, int ny, int nz, bool f64, int max_smem, int kind, MixedPlan* m)

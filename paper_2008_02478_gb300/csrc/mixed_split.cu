@@ -3,10 +3,11 @@
 // ml_mixed_y.cu), the z stage in place on Y, y inverses.  For meshes whose plane
 // does not fit one CTA's shared memory, or whose planes leave SMs idle, where
 // the power-of-two lengths pad most (mixed_pays): the z stage, the transforms of
-// plane_conv.cuh, reaches a third of the copy rate (loads' latency at 12 to 20
-// warps per SM), the power-of-two one two thirds.  Evaluations, before -> now: 160 x 640 x 12
-// 238 -> 149 us, 86 x 705 x 8 87 -> 53, 39 x 143 x 23 56 -> 32, 283 x 269 x 24 412 -> 290,
-// 545 x 836 x 6 525 -> 436 (power-of-two passes), 160 x 160 x 20 69 -> 62 (planes).
+// plane_conv.cuh, reaches a third to a half of the copy rate (loads' latency at
+// 8 to 20 warps per SM), the power-of-two one two thirds.  Evaluations, before ->
+// now: 160 x 640 x 12 238 -> 131 us, 86 x 705 x 8 87 -> 53, 39 x 143 x 23 56 -> 32,
+// 283 x 269 x 24 412 -> 287, 48 x 512 x 32 140 -> 86, 545 x 836 x 6 525 -> 436 (power-of-two
+// passes), 160 x 160 x 20 69 -> 62 (planes).
 #include "bulk_async.cuh"
 #include "ml_mixed.cuh"
 #include "plane_conv.cuh"
@@ -16,21 +17,22 @@ namespace boris {
 namespace {
 
 // Four warps per CTA, the items of all kx side by side (545 x 836 x 6: 126 us with
-// those of one kx side by side, now 107).  HZ 16 to 24: TK bins ky' of one kx and
-// their mirrors go through shared memory in rows of 256 consecutive bytes,
-// [line][TK | 8 | TK] (the gap keeps a bin and its mirror in different banks);
-// with other lengths each warp reads and writes one item's columns in 32- to
-// 64-byte pieces (staged against direct: 80 x 897 x 23 121 and 171 us, 128 x 200 x 20 28
-// and 35; 545 x 836 x 6 155 and 120, 300 x 400 x 8 47 and 35).  The kernel rows of the
-// tile come with the columns: read where they are used, they were what the
-// warps waited for (283 x 269 x 24: 153 us, now 122; 80 x 897 x 23 115, now 90).
+// those of one kx side by side, now 107).  From HZ 12 on TK bins ky' of one kx,
+// their mirrors and their kernel rows go through shared memory in rows of 256
+// consecutive bytes, columns as [line][TK | 8 | TK] (the gap keeps a bin and its
+// mirror in different banks): read where they are used, the kernel rows were what
+// the warps waited for (direct against staged: 160 x 640 x 12 59 and 42 us, 160 x 160
+// x 20 25 and 23, 283 x 269 x 24 153 and 122, 55 x 767 x 26 170 and 80).  To HZ 8 each
+// warp reads and writes one item's columns in 64-byte pieces (256 x 256 x 8 12.2
+// and 15.5, 700 x 700 x 5 89 and 104).
 constexpr int TK = 32, ZLS = 2 * TK + 8;
 constexpr int KP = 44;  // pitch of a staged kernel row: the rows of four residues start four pairs apart mod 16
-constexpr bool z_staged(int HZ) { return HZ >= 16 && HZ <= 24; }
+constexpr bool z_staged(int HZ) { return HZ >= 12; }
 
 template <int HZ, int RES>
-__global__ void __launch_bounds__(128, z_staged(HZ) ? 3 : HZ <= 12 ? 5 : 2) z_conv_kernel(int H, int nz, int kyp, int nkz, float2* __restrict__ Y,
-                                                     const float2* __restrict__ K, const float2* __restrict__ twz)
+__global__ void __launch_bounds__(128, HZ <= 12 ? 5 : HZ == 32 ? 2 : 3)
+    z_conv_kernel(int H, int nz, int kyp, int nkz, float2* __restrict__ Y, const float2* __restrict__ K,
+                  const float2* __restrict__ twz)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int KB = 16 / RES;
@@ -70,7 +72,7 @@ template <int HZ>
 cudaError_t z_launch(const MixedPlan& m, float2* Y, const float2* K, cudaStream_t st)
 {
     constexpr int RES = HZ <= 8 ? 2 : 4;
-    const size_t smem = z_staged(HZ) ? ((size_t)3 * m.nz * ZLS + (size_t)3 * m.nkz * KP) * sizeof(float2) : 0;  // 68 KB at most
+    const size_t smem = z_staged(HZ) ? ((size_t)3 * m.nz * ZLS + (size_t)3 * m.nkz * KP) * sizeof(float2) : 0;  // 90 KB at most
     const cudaError_t e = cudaFuncSetAttribute(z_conv_kernel<HZ, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int tiles = z_staged(HZ) ? m.y.H / TK + 1 : (m.y.H * RES / 16 + 4) / 4;
