@@ -68,6 +68,7 @@ cudaError_t launch_plane_conv(const MixedPlan& m, typename Cx<T>::t* X, const ty
 // The passes (mixed_split.cu); g, tw: the geometry and twiddles of the 1024-point kernels
 cudaError_t launch_mixed_y(const MixedPlan& m, const Geometry& g, float2* X, float2* Y, const float2* tw, cudaStream_t st,
                            bool forward);
+cudaError_t mixed_z_prepare(const MixedPlan& m);  // (once, at plan creation)
 cudaError_t launch_mixed_z(const MixedPlan& m, float2* Y, const float2* K, cudaStream_t st);
 
 // per-type, per-class pieces (one translation unit each)

@@ -242,8 +242,9 @@ static cudaError_t prepare_t(const MixedPlan& m)
 cudaError_t mixed_prepare(const MixedPlan& m, bool f64)
 {
     if (m.split) {
-        const cudaError_t e = x_set_attr<float>(m);
-        return e == cudaSuccess ? line_y_prepare(m) : e;
+        cudaError_t e = x_set_attr<float>(m);
+        if (e == cudaSuccess) e = line_y_prepare(m);
+        return e == cudaSuccess ? mixed_z_prepare(m) : e;
     }
     return f64 ? prepare_t<double>(m) : prepare_t<float>(m);
 }

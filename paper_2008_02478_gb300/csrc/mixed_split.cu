@@ -69,26 +69,54 @@ __global__ void __launch_bounds__(128, HZ <= 12 ? 5 : HZ == 32 ? 2 : 3)
 }
 
 template <int HZ>
+constexpr int z_res = HZ <= 8 ? 2 : 4;
+
+// Shared memory of a CTA for nz planes and nkz kernel rows, 90 KB at most.
+constexpr size_t z_smem(int HZ, int nz, int nkz)
+{
+    return z_staged(HZ) ? ((size_t)3 * nz * ZLS + (size_t)3 * nkz * KP) * sizeof(float2) : 0;
+}
+
+// The shared-memory limit belongs to the kernel, which plans of every nz with this
+// HZ share: it is set to what the largest nz takes, so no plan lowers it for another.
+template <int HZ>
+cudaError_t z_prepare()
+{
+    return cudaFuncSetAttribute(z_conv_kernel<HZ, z_res<HZ>>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)z_smem(HZ, HZ, HZ + 1));
+}
+
+template <int HZ>
 cudaError_t z_launch(const MixedPlan& m, float2* Y, const float2* K, cudaStream_t st)
 {
-    constexpr int RES = HZ <= 8 ? 2 : 4;
-    const size_t smem = z_staged(HZ) ? ((size_t)3 * m.nz * ZLS + (size_t)3 * m.nkz * KP) * sizeof(float2) : 0;  // 90 KB at most
-    const cudaError_t e = cudaFuncSetAttribute(z_conv_kernel<HZ, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    constexpr int RES = z_res<HZ>;
     const int tiles = z_staged(HZ) ? m.y.H / TK + 1 : (m.y.H * RES / 16 + 4) / 4;
-    z_conv_kernel<HZ, RES><<<dim3(m.x.H + 1, tiles), 128, smem, st>>>(m.y.H, m.nz, m.kyp, m.nkz, Y, K,
-                                                                             (const float2*)m.twz);
+    z_conv_kernel<HZ, RES><<<dim3(m.x.H + 1, tiles), 128, z_smem(HZ, m.nz, m.nkz), st>>>(m.y.H, m.nz, m.kyp, m.nkz, Y, K,
+                                                                                        (const float2*)m.twz);
     return cudaGetLastError();
 }
 
 }  // namespace
+
+#define Z_SIZES(Z) Z(2) Z(4) Z(6) Z(8) Z(12) Z(16) Z(20) Z(24) Z(32)
+
+cudaError_t mixed_z_prepare(const MixedPlan& m)
+{
+    switch (m.HZ) {
+#define Z(h) \
+    case h: return z_prepare<h>();
+        Z_SIZES(Z)
+#undef Z
+    }
+    return cudaErrorInvalidValue;
+}
 
 cudaError_t launch_mixed_z(const MixedPlan& m, float2* Y, const float2* K, cudaStream_t st)
 {
     switch (m.HZ) {
 #define Z(h) \
     case h: return z_launch<h>(m, Y, K, st);
-        Z(2) Z(4) Z(6) Z(8) Z(12) Z(16) Z(20) Z(24) Z(32)
+        Z_SIZES(Z)
 #undef Z
     }
     return cudaErrorInvalidValue;
