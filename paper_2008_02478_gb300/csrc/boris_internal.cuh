@@ -21,6 +21,12 @@ inline int padded_len(int n)
     while (p < 2 * n - 1) p <<= 1;
     return p;
 }
+// Dynamic shared memory that a CTA without static shared memory can have.  A kernel's
+// limit belongs to the kernel, not to a plan: where the amount differs from plan to
+// plan it is always set to this, so that no host thread lowers it between another's
+// setting and launch.
+constexpr int SMEM_MAX = 227 * 1024;
+
 inline int ilog2(int v)
 {
     int l = 0;

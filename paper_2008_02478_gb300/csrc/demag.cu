@@ -349,7 +349,7 @@ static cudaError_t launch_r2c_ty(const Geometry& g, const T* M, const T* ms_map,
                                  typename Cx<T>::t* X, const typename Cx<T>::t* tw, cudaStream_t st)
 {
     const size_t smem = (size_t)(TY / 2) * g.px * sizeof(typename Cx<T>::t);
-    cudaError_t e = cudaFuncSetAttribute(x_r2c_kernel<T, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(x_r2c_kernel<T, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
     if (e != cudaSuccess) return e;
     dim3 grid((g.ny + TY - 1) / TY, g.nz, 3);
     x_r2c_kernel<T, TY><<<grid, 256, smem, st>>>(g, M, ms_map, ms_scale, X, tw);
@@ -377,7 +377,7 @@ static cudaError_t launch_c2r_ty(const Geometry& g, const typename Cx<T>::t* X, 
                                  const typename Cx<T>::t* tw, cudaStream_t st)
 {
     const size_t smem = (size_t)(TY / 2) * g.px * sizeof(typename Cx<T>::t);
-    cudaError_t e = cudaFuncSetAttribute(x_c2r_kernel<T, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(x_c2r_kernel<T, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
     if (e != cudaSuccess) return e;
     dim3 grid((g.ny + TY - 1) / TY, g.nz, 3);
     x_c2r_kernel<T, TY><<<grid, 256, smem, st>>>(g, X, H, tw);
@@ -460,7 +460,7 @@ bool choose_yz_schedule(const Geometry& g, int max_smem, YZSchedule* out)
 template <typename T, int CC>
 static cudaError_t set_attr_cc(const YZSchedule& sc)
 {
-    cudaError_t e = cudaFuncSetAttribute(yz_conv_kernel<T, CC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sc.smem);
+    cudaError_t e = cudaFuncSetAttribute(yz_conv_kernel<T, CC>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
     if (e != cudaSuccess) return e;
     if (CC > 8) e = cudaFuncSetAttribute(yz_conv_kernel<T, CC>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
@@ -470,7 +470,7 @@ template <typename T, int CC>
 static cudaError_t launch_yz_cc(const Geometry& g, const YZSchedule& sc, typename Cx<T>::t* X, const T* K,
                                 const typename Cx<T>::t* tw, cudaStream_t st)
 {
-    // the attributes are per function: set them for this launch's shared memory
+    // the attributes are per function
     cudaError_t e = set_attr_cc<T, CC>(sc);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};

@@ -333,7 +333,7 @@ cudaError_t launch_split(const Geometry& g, typename Cx<T>::t* X, typename Cx<T>
     if (part != 1 && y2048_ok<T>(g, 227 * 1024)) return launch_y_2048<T>(g, X, Y, tw, st, part == 0);
     if (part != 1 && y4096_ok<T>(g, 227 * 1024)) return launch_y_4096<T>(g, X, Y, tw, st, part == 0);
     if (part == 0) {
-        e = cudaFuncSetAttribute(y_fwd_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ys);
+        e = cudaFuncSetAttribute(y_fwd_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
         if (e != cudaSuccess) return e;
         y_fwd_kernel<T><<<ygrid, 256, ys, st>>>(g, X, Y, tw);
         return cudaGetLastError();
@@ -354,7 +354,7 @@ cudaError_t launch_split(const Geometry& g, typename Cx<T>::t* X, typename Cx<T>
         default: return cudaErrorInvalidValue;
         }
     }
-    e = cudaFuncSetAttribute(y_inv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ys);
+    e = cudaFuncSetAttribute(y_inv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
     if (e != cudaSuccess) return e;
     y_inv_kernel<T><<<ygrid, 256, ys, st>>>(g, Y, X, tw);
     return cudaGetLastError();

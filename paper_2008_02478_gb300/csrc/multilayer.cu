@@ -679,7 +679,7 @@ cudaError_t ml_mix(const Geometry& g, int Z, float2* Y, const float* K, const in
         const int ntile = g.py / 64 + 1, nwork = ntile * g.nkx;
         const int G = std::min(nwork, (variant - 1) * nsm);
 #define ML_V2(P)                                                                                             \
-    e = cudaFuncSetAttribute(ml_mix_v2_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);   \
+    e = cudaFuncSetAttribute(ml_mix_v2_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);   \
     if (e != cudaSuccess) return e;                                                                          \
     ml_mix_v2_kernel<P><<<G, 256, smem, st>>>(g, Z, Y, K, pcode, inv_hz, ntile, nwork);                      \
     return cudaGetLastError();
@@ -700,11 +700,11 @@ cudaError_t ml_mix(const Geometry& g, int Z, float2* Y, const float* K, const in
     const size_t smem = staged ? smem_s : (size_t)Z * 3 * 64 * sizeof(float2) + (size_t)Z * Z * sizeof(int);
 #define ML_MIX(P)                                                                                              \
     if (staged) {                                                                                              \
-        e = cudaFuncSetAttribute(ml_mix_staged_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+        e = cudaFuncSetAttribute(ml_mix_staged_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX); \
         if (e != cudaSuccess) return e;                                                                        \
         ml_mix_staged_kernel<P><<<grid, 256, smem, st>>>(g, Z, Y, K, kyp, pairs, inv_hz);                      \
     } else {                                                                                                   \
-        e = cudaFuncSetAttribute(ml_mix_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);     \
+        e = cudaFuncSetAttribute(ml_mix_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);     \
         if (e != cudaSuccess) return e;                                                                        \
         ml_mix_kernel<P><<<grid, 256, smem, st>>>(g, Z, Y, K, kyp, pairs, inv_hz);                             \
     }                                                                                                          \

@@ -253,7 +253,7 @@ cudaError_t run_axis_n(const void* in, bool in_real, double2* out, int axis, int
     if (NL < 1) NL = 1;
     if (NL > 32) NL = 32;
     const size_t smem = (size_t)NL * P * sizeof(double2);
-    cudaError_t e = cudaFuncSetAttribute(axis_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(axis_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
     if (e != cudaSuccess) return e;
     const int dims[3] = {d0, d1, d2};
     const int oa = axis == 0 ? 1 : 0, ob = axis == 2 ? 1 : 2;

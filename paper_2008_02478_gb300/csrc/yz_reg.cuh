@@ -202,7 +202,7 @@ cudaError_t launch_yz_reg_t(const Geometry& g, size_t smem, typename Cx<T>::t* X
                             const typename Cx<T>::t* tw, cudaStream_t st)
 {
     cudaError_t e = cudaFuncSetAttribute(yz_conv_reg_kernel<T, CC, HZ, NT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
     if (e != cudaSuccess) return e;
     if (CC > 8) {
         e = cudaFuncSetAttribute(yz_conv_reg_kernel<T, CC, HZ, NT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
