@@ -187,10 +187,10 @@ int boris_demag_apply_f64(boris_plan p, const double* M, double* Hd);
  *   workspace is a fixed 32 MiB device array inside the library (held by every
  *   GPU that loads the library until the process exits), so it accepts meshes
  *   whose spectral workspace - (px/2 + 1) * 3 * nz * ny * 8 bytes, plus
- *   (px/2 + 1) * py * 3 * nz * 8 bytes when the plan chose the split y-z
- *   schedule (on kinds 3 and 4: where the split schedule serves the mesh),
- *   px and py powers of two - fits in 32 MiB, and returns BORIS_ERR_UNSUPPORTED_SIZE for
- *   larger ones.  The plan (made at set-up)
+ *   (px/2 + 1) * py * 3 * nz * 8 bytes when the plan runs the y-z part in
+ *   passes (schedule kinds 2 and 4), px and py those of boris_plan_padded -
+ *   fits in 32 MiB, and returns BORIS_ERR_UNSUPPORTED_SIZE for larger ones.
+ *   The plan (made at set-up)
  *   still supplies the kernel spectrum.  The plan's device must be current.
  *   The first call on a device looks up the array's device address; make that
  *   first call before any stream capture.  All calls share the one array:

@@ -271,7 +271,6 @@ struct PlanView {
     bool oersted;  // Oersted plan: its spectrum is the curl kernel, not the demag tensor
     const MixedPlan* mixed;  // mixed-radix path (schedule kind 3), else NULL
     bool mixed_x1024;        // with the power-of-two x passes
-    size_t noalloc_need;     // its workspace need in boris_demag_apply_noalloc
 };
 // Number of kernel classes timed by the plan's profiler.
 constexpr int NPROF = 9;

@@ -85,7 +85,6 @@ struct boris_plan_s {
     bool mixed_x1024 = false;  // its x passes are the power-of-two ones (px 1024, 2048)
     void* mtw = nullptr;
     unsigned short* mpos = nullptr;
-    size_t noalloc_need = 0;  // bytes boris_demag_apply_noalloc asks for on this mesh
     // column-major padded spectrum [kx][ky][c][z] of the split schedule
     void* Y = nullptr;
     // LLG workspace (allocated on first use)
@@ -892,7 +891,6 @@ bool plan_view(boris_plan p, PlanView* v)
     v->oersted = p->oersted;
     v->mixed = p->mixed ? &p->mp : nullptr;
     v->mixed_x1024 = p->mixed_x1024;
-    v->noalloc_need = p->noalloc_need;
     return true;
 }
 }  // namespace boris
@@ -983,10 +981,6 @@ static int plan_create(int nx, int ny, int nz, double dx, double dy, double dz, 
     }
     int max_smem = 0;
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
-    // workspace of boris_demag_apply_noalloc on this mesh (power-of-two lengths)
-    const bool split_fits = p->f64 ? split_supported<double>(g, max_smem) : split_supported<float>(g, max_smem);
-    p->noalloc_need = (((size_t)g.nkx * 3 * nz * ny * sizeof(float2) + 255) & ~(size_t)255) +
-                      (split_fits ? (size_t)g.nkx * g.py * 3 * nz * sizeof(float2) : 0);
     // Mixed-radix lengths with the whole kx plane in one CTA's shared memory,
     // or y, z and y passes, where they pay (mixed_pays) and no switch pins another
     // schedule; BORIS_YZ_KIND=3 and 4 take the one and the other wherever they can.
@@ -997,8 +991,7 @@ static int plan_create(int nx, int ny, int nz, double dx, double dy, double dz, 
     for (const char* v : {"BORIS_YZ_CLUSTER", "BORIS_YZ_THREADS", "BORIS_YZ_QC", "BORIS_YZ_TMA"})
         pinned |= std::getenv(v) != nullptr;
     if (const char* sf = std::getenv("BORIS_FUSE_STAGE")) pinned |= std::atoi(sf) == 1;
-    if (!pinned && mixed_plan_shape(nx, ny, nz, p->f64, max_smem, fk, &p->mp) && (forced || mixed_pays(p->mp, p->f64, g)) &&
-        (!p->mp.split || split_fits)) {  // (noalloc_need has no second workspace otherwise)
+    if (!pinned && mixed_plan_shape(nx, ny, nz, p->f64, max_smem, fk, &p->mp) && (forced || mixed_pays(p->mp, p->f64, g))) {
         p->mixed = true;
         Geometry& mg = p->g;
         mg.px = 2 * p->mp.x.H;
@@ -1026,7 +1019,7 @@ static int plan_create(int nx, int ny, int nz, double dx, double dy, double dz, 
     int ncand = 0;
     if (p->f64) yz_candidates<double>(g, max_smem, cand, &ncand);
     else yz_candidates<float>(g, max_smem, cand, &ncand);
-    const bool split_ok = split_fits;
+    const bool split_ok = p->f64 ? split_supported<double>(g, max_smem) : split_supported<float>(g, max_smem);
     if (split_ok && ncand < 14) {
         cand[ncand++] = YZSchedule{2, 2, 0, 0, 0};
         if (!p->f64) cand[ncand++] = YZSchedule{2, 3, 0, 0, 0};

@@ -75,10 +75,11 @@ extern "C" int boris_demag_apply_noalloc(boris_plan p, const float* M, float* Hd
         return BORIS_ERR_INVALID_ARG;
     }
     const size_t xbytes = (size_t)v.g.nkx * 3 * v.g.nz * v.g.ny * sizeof(float2);
-    // the split y-z schedule also needs the column-major padded spectrum
-    const size_t ybytes = v.yz.kind == 2 ? (size_t)v.g.nkx * v.g.py * 3 * v.g.nz * sizeof(float2) : 0;
+    // the schedules in three passes also need the column-major padded spectrum
+    const bool passes = v.mixed ? v.mixed->split : v.yz.kind == 2;
+    const size_t ybytes = passes ? (size_t)v.g.nkx * v.g.py * 3 * v.g.nz * sizeof(float2) : 0;
     const size_t xoff = (xbytes + 255) & ~(size_t)255;
-    const size_t need = v.mixed ? v.noalloc_need : xoff + ybytes;
+    const size_t need = xoff + ybytes;
     if (need > NOALLOC_SCRATCH_BYTES) {
         set_error("mesh spectrum needs " + std::to_string(need) + " bytes; the allocation-free workspace holds " +
                   std::to_string(NOALLOC_SCRATCH_BYTES) + " bytes (use boris_demag_apply)");
