@@ -171,7 +171,18 @@ bool mixed_pays(const MixedPlan& m, bool f64, const Geometry& pow2)
         // x 16: 490 us) against 2.2e-4 to 3.2e-4 over all planes (564 us)
         const double w = 3.0 * m.nz * 2.0 * m.y.H, per_sm = (m.x.H + 152) / 152;
         const double c = m.HZ == 1 ? 25e-3 : m.HZ <= 4 ? 31e-3 : m.HZ <= 8 ? 36e-3 : 40e-3;
-        return per_sm * w * c <= std::max(15.0, all * (m.HZ == 1 ? 2.2e-4 : m.HZ <= 4 ? 2.4e-4 : 3.2e-4));
+        // a tenth more from three planes per SM on where the z axis saves nothing and a plane
+        // is large: there the x passes cost more than the 1024-point ones, too (evaluations,
+        // this path against the other: 387 x 51 x 32 2642 and 2298 us, 457 x 463 x 4 2088 and 1770)
+        const double edge = per_sm >= 3 && 2 * m.HZ == pow2.pz && w >= 2500 ? 1.1 : 1.0;
+        // the shortest calls take as long either way up to HZ 4; beyond, the chain of the
+        // z stage is longer here (49 x 3 x 18 86 and 55 us, 51 x 7 x 6 66 and 51)
+        const double least = m.HZ <= 4 ? 15.0 : 0.0;
+        // HZ 32 computes all 32 planes whatever nz is: 25 us and 46e-3 per point of them a plane,
+        // against 130 us and 3.3e-4 (919 x 8 x 32 798 and 662 us, 214 x 56 x 25 1167 and 1068)
+        if (m.HZ > 24 && per_sm * (25.0 + 46e-3 * 96.0 * 2.0 * m.y.H) > 0.98 * (130.0 + 3.3e-4 * 96.0 * pow2.py * pow2.nkx))
+            return false;
+        return edge * per_sm * w * c <= std::max(least, all * (m.HZ == 1 ? 2.2e-4 : m.HZ <= 4 ? 2.4e-4 : 3.2e-4));
     }
     // their x passes take longer on short rows, per row and evaluation 3.8e-3 us to
     // 128 points (37 x 398 x 16: 35 against 11 us), 2e-3 with 256, 0.6e-3 with 512

@@ -1,0 +1,28 @@
+"""Meshes on which the mixed-radix schedules measured slower than the power-of-two ones are not given
+to them, and the ones they were made for are."""
+import pytest
+
+from tests.gpu_util import torch_cuda
+
+pytestmark = pytest.mark.gpu
+
+
+def kind(n, fp64):
+    torch_cuda()
+    from paper_2008_02478_gb300.binding import Plan
+    plan = Plan(*n, 3e-9, 3e-9, 3e-9, fp64=fp64)
+    k = plan.schedule()[0]
+    plan.close()
+    return k
+
+
+@pytest.mark.parametrize("n", [(387, 51, 32), (457, 463, 4), (393, 479, 2), (389, 28, 15), (420, 30, 14), (415, 25, 29),
+                               (919, 8, 32),
+                               (214, 56, 25), (49, 3, 18), (34, 3, 20), (51, 7, 6), (64, 4, 11)])
+def test_fp64_meshes_left_to_powers_of_two(n):
+    assert kind(n, True) < 3
+
+
+@pytest.mark.parametrize("n", [(128, 128, 16), (32, 70, 1), (59, 21, 3), (407, 111, 18), (428, 4, 13), (186, 32, 29)])
+def test_fp64_meshes_on_mixed_lengths(n):
+    assert kind(n, True) == 3
