@@ -188,12 +188,20 @@ bool mixed_pays(const MixedPlan& m, bool f64, const Geometry& pow2)
     // 128 points (37 x 398 x 16: 35 against 11 us), 2e-3 with 256, 0.6e-3 with 512
     const double x = (double)m.y.n * m.nz * (pow2.px <= 128 ? 3.8e-3 : pow2.px == 256 ? 2e-3 : pow2.px == 512 ? 0.6e-3 : 0.0);
     if (m.split) {
+        // few short x lines: the five launches take 25 to 35 us whatever the points, the
+        // power-of-two schedules less up to so many points of a plane (evaluations: 3 x 395 x 4
+        // 31 and 21 us, 4 x 42 x 28 31 and 23, 6 x 815 x 2 35 and 32; 4 x 2000 x 16 and more 1.1 to 1.6 times
+        // the other way)
+        if (pow2.px <= 16 && pow2.py < 4096 && (long)pow2.py * pow2.pz < (pow2.px <= 8 ? 65536 : 16384)) return false;
         // 20 us (10 with 33 planes: 27 x 137 x 26 23) plus 7.7e-6 for a full z axis (320 x 388 x 16: 200), more with padding in z
         // (283 x 269 x 24: 370), an eighth more from 2048 points in y (160 x 640 x 12: 205);
         // taken from 8 % less on (197 x 769 x 10, not taken: 227 against 306)
         const double pad = 0.6 + 0.2 * pow2.pz / m.nz;
         return passes_us(m) <= 0.92 * ((pow2.px <= 64 ? 10.0 : 20.0) + all * 7.7e-6 * pad) * (pow2.py >= 2048 ? 1.12 : 1.0) + x;
     }
+    // on at most five planes the long z stage takes longer than those of the cluster
+    // schedules (3 x 16 x 27 21 and 18 us, 2 x 59 x 15 23 and 21)
+    if ((pow2.px <= 8 && m.HZ > 24) || (pow2.px <= 4 && m.HZ > 12)) return false;
     // 8.8e-6 plus 6 us, 16 us at least and 25 from HZ 12 and 128 x points on (256 x 256 x 16: 55 us
     // against 75 in planes; 27 x 137 x 26, 33 planes of 25 k points: 22 against 51; 34 x 88
     // x 22: 31 against 22); with fewer points in x, too, 15 % more

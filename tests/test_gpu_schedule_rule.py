@@ -26,3 +26,15 @@ def test_fp64_meshes_left_to_powers_of_two(n):
 @pytest.mark.parametrize("n", [(128, 128, 16), (32, 70, 1), (59, 21, 3), (407, 111, 18), (428, 4, 13), (186, 32, 29)])
 def test_fp64_meshes_on_mixed_lengths(n):
     assert kind(n, True) == 3
+
+
+@pytest.mark.parametrize("n", [(3, 395, 4), (4, 720, 2), (2, 54, 31), (4, 42, 28), (4, 52, 16), (2, 931, 4), (6, 815, 2), (5, 404, 3),
+                               (3, 16, 27), (2, 59, 15)])
+def test_few_lines_left_to_powers_of_two(n):
+    assert kind(n, False) < 3
+
+
+@pytest.mark.parametrize("n,k", [((32, 32, 4), 3), ((16, 16, 27), 3), ((4, 39, 13), 3), ((4, 1394, 3), 4), ((3, 1500, 16), 4), ((5, 500, 30), 4),
+                                 ((12, 300, 20), 4), ((160, 640, 12), 4)])
+def test_fp32_meshes_on_mixed_lengths(n, k):
+    assert kind(n, False) == k
