@@ -409,7 +409,8 @@ int boris_plan_padded(boris_plan p, int out[3]);
  * split into y-forward / z-convolution / y-inverse kernels, 3: one CTA per kx
  * plane on mixed-radix lengths, where a padded plane fits a CTA's shared
  * memory, 4: y, z and y passes on mixed-radix lengths (FP32, nz > 1); 3 and 4
- * are taken without timing by a rule on the sizes; multi-mesh plans
+ * are taken by a rule on the sizes, in FP32 timed against kind 2 where its
+ * estimates are close; multi-mesh plans
  * report kind 2 with out[2] the inter-plane sum variant: 0 one CTA per tile,
  * 1 staged rows, 2 or 3 one persistent launch with 1 or 2 CTAs per SM).
  * Kinds 0, 1, 3 and 4:

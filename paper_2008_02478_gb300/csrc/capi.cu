@@ -899,8 +899,55 @@ extern "C" {
 
 const char* boris_last_error(void) { return g_last_error.c_str(); }
 
+// pow2_only: the split power-of-two schedules, chosen among them by timing, with zeros
+// in place of the kernel spectrum (build_pow2_spectrum fills it in)
 static int plan_create(int nx, int ny, int nz, double dx, double dy, double dz, unsigned flags, void* cuda_stream,
-                       boris_plan* out, const int* images);
+                       boris_plan* out, const int* images, bool pow2_only = false);
+
+// Kernel spectrum of a power-of-two plan, and its column-major copy where the plan has one.
+static int build_pow2_spectrum(boris_plan p)
+{
+    cudaError_t ce = build_kernel_spectrum(p->g, p->dx, p->dy, p->dz, 40.0, p->K, p->f64, p->tw64, p->stream, p->images);
+    if (ce != cudaSuccess) return fail(BORIS_ERR_CUDA, std::string("kernel spectrum: ") + cudaGetErrorString(ce));
+    if (p->K2 && (ce = zconv_res_build_k2(p->g, (const float*)p->K, (float2*)p->K2, p->stream)) != cudaSuccess)
+        return fail(BORIS_ERR_CUDA, std::string("kernel spectrum copy: ") + cudaGetErrorString(ce));
+    if ((ce = cudaStreamSynchronize(p->stream)) != cudaSuccess)
+        return fail(BORIS_ERR_CUDA, std::string("kernel spectrum: ") + cudaGetErrorString(ce));
+    return BORIS_OK;
+}
+
+// Whether FP32 plan b evaluates the field faster than a, by 3 % or more: the shortest of three
+// runs of two evaluations each, in turn, on a field of zeros.  False where there is no room for it.
+static bool evaluates_faster(boris_plan b, boris_plan a)
+{
+    float* f = nullptr;
+    const size_t n3 = 3 * (size_t)a->g.nx * a->g.ny * a->g.nz, h = (n3 + 3) / 4 * 4;
+    if (cudaMallocAsync((void**)&f, (h + n3) * sizeof(float), a->stream) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    bool ok = cudaMemsetAsync(f, 0, (h + n3) * sizeof(float), a->stream) == cudaSuccess &&
+              cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess;
+    float best[2] = {1e30f, 1e30f};
+    const long long launches[2] = {a->launches, b->launches};
+    for (int r = 0; r < 8 && ok; r++) {  // (the first run of each warms up)
+        boris_plan p = r & 1 ? b : a;
+        cudaEventRecord(e0, p->stream);
+        for (int k = 0; k < 2 && ok; k++) ok = demag_apply_t<float>(p, f, nullptr, 1.0f, f + h) == BORIS_OK;
+        cudaEventRecord(e1, p->stream);
+        float ms = 0.f;
+        ok = ok && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess;
+        if (r >= 2) best[r & 1] = std::min(best[r & 1], ms);
+    }
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
+    cudaFreeAsync(f, a->stream);
+    a->launches = launches[0];
+    b->launches = launches[1];
+    if (!ok) cudaGetLastError();
+    return ok && best[1] < 0.97f * best[0];
+}
 
 int boris_demag_plan(int nx, int ny, int nz, double dx, double dy, double dz, unsigned flags, void* cuda_stream,
                      boris_plan* out)
@@ -918,7 +965,7 @@ int boris_demag_plan_pbc(int nx, int ny, int nz, double dx, double dy, double dz
 }
 
 static int plan_create(int nx, int ny, int nz, double dx, double dy, double dz, unsigned flags, void* cuda_stream,
-                       boris_plan* out, const int* images)
+                       boris_plan* out, const int* images, bool pow2_only)
 {
     if (!out) return fail(BORIS_ERR_INVALID_ARG, "out is NULL");
     *out = nullptr;
@@ -987,11 +1034,11 @@ static int plan_create(int nx, int ny, int nz, double dx, double dy, double dz, 
     const char* kind = std::getenv("BORIS_YZ_KIND");
     const int fk = kind ? std::atoi(kind) : 0;
     const bool forced = fk == 3 || fk == 4;
-    bool pinned = tc != 0 || (kind && !forced);
+    bool pinned = pow2_only || tc != 0 || (kind && !forced), close = false;
     for (const char* v : {"BORIS_YZ_CLUSTER", "BORIS_YZ_THREADS", "BORIS_YZ_QC", "BORIS_YZ_TMA"})
         pinned |= std::getenv(v) != nullptr;
     if (const char* sf = std::getenv("BORIS_FUSE_STAGE")) pinned |= std::atoi(sf) == 1;
-    if (!pinned && mixed_plan_shape(nx, ny, nz, p->f64, max_smem, fk, &p->mp) && (forced || mixed_pays(p->mp, p->f64, g))) {
+    if (!pinned && mixed_plan_shape(nx, ny, nz, p->f64, max_smem, fk, &p->mp) && (forced || mixed_pays(p->mp, p->f64, g, &close))) {
         p->mixed = true;
         Geometry& mg = p->g;
         mg.px = 2 * p->mp.x.H;
@@ -1012,6 +1059,15 @@ static int plan_create(int nx, int ny, int nz, double dx, double dy, double dz, 
         }
         p->yz = p->mp.split ? YZSchedule{4, 1, 0, 128, 0} : YZSchedule{3, 1, 0, p->mp.threads, p->mp.smem};
         if ((rc = mixed_setup(p))) return bail(rc);
+        // where the estimates are close: the faster of the two, as timed; the power-of-two
+        // spectrum is built only where it is taken
+        boris_plan other = nullptr;
+        if (close && plan_create(nx, ny, nz, dx, dy, dz, flags, cuda_stream, &other, images, true) == BORIS_OK) {
+            if (evaluates_faster(other, p) && build_pow2_spectrum(other) == BORIS_OK) std::swap(p, other);
+            boris_plan_destroy(other);
+        } else if (close) {
+            cudaGetLastError();  // no room for both
+        }
         *out = p;
         return BORIS_OK;
     }
@@ -1032,6 +1088,14 @@ static int plan_create(int nx, int ny, int nz, double dx, double dy, double dz, 
             cand[ncand++] = YZSchedule{2, 4, 3, 0, 0};
             cand[ncand++] = YZSchedule{2, 3, 3, 0, 0};
         }
+    }
+    // where the estimates are close the split schedule is the fastest of them, or the mixed
+    // lengths are anyway (1082 meshes); timing the others took most of a plan's making
+    if (pow2_only && split_ok) {
+        int m = 0;
+        for (int i = 0; i < ncand; i++)
+            if (cand[i].kind == 2) cand[m++] = cand[i];
+        ncand = m;
     }
     if (tc) {
         // the tensor-core z stage runs inside the split schedule only
@@ -1103,9 +1167,9 @@ static int plan_create(int nx, int ny, int nz, double dx, double dy, double dz, 
     const size_t kelems = (size_t)g.nkx * g.kyh * g.krow;
     const size_t esz = p->f64 ? sizeof(double) : sizeof(float);
     if ((rc = dev_alloc(p, &p->K, kelems * esz))) return bail(rc);
-    const double rs = 40.0;
-    ce = build_kernel_spectrum(g, dx, dy, dz, rs, p->K, p->f64, p->tw64, p->stream, p->images);
-    if (ce != cudaSuccess) return bail(fail(BORIS_ERR_CUDA, std::string("kernel spectrum: ") + cudaGetErrorString(ce)));
+    if (!pow2_only) rc = build_pow2_spectrum(p);
+    else if (cudaMemsetAsync(p->K, 0, kelems * esz, p->stream) != cudaSuccess) rc = fail(BORIS_ERR_CUDA, "kernel spectrum");
+    if (rc) return bail(rc);
     // spectral workspace
     const size_t xelems = (size_t)g.nkx * 3 * g.nz * g.ny;
     if ((rc = dev_alloc(p, &p->X, xelems * 2 * esz))) return bail(rc);

@@ -48,8 +48,9 @@ constexpr int ZTAB = 256;
 // Whether the mesh runs on this path (host rule); fills the axis plans.
 // kind 3 or 4: the plane kernel or the passes wherever possible, 0: the faster one
 bool mixed_plan_shape(int nx, int ny, int nz, bool f64, int max_smem, int kind, MixedPlan* m);
-// Whether it is the faster path there (pow2: the power-of-two geometry of the same mesh).
-bool mixed_pays(const MixedPlan& m, bool f64, const Geometry& pow2);
+// Whether it is the faster path there by the estimates (pow2: the power-of-two geometry of
+// the same mesh); *close: they can be wrong by as much as they differ, so time both.
+bool mixed_pays(const MixedPlan& m, bool f64, const Geometry& pow2, bool* close);
 // Host tables of the plan, concatenated: [twx | twy | twz], positions [posx | posy]
 size_t mixed_tw_entries(const MixedPlan& m, size_t* oy, size_t* oz);
 void mixed_tw_fill(const MixedPlan& m, double2* out);

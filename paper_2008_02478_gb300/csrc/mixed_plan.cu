@@ -162,8 +162,9 @@ bool mixed_plan_shape(int nx, int ny, int nz, bool f64, int max_smem, int kind, 
     return true;
 }
 
-bool mixed_pays(const MixedPlan& m, bool f64, const Geometry& pow2)
+bool mixed_pays(const MixedPlan& m, bool f64, const Geometry& pow2, bool* close)
 {
+    *close = false;
     // The power-of-two schedules spread all points over the chip but have more of them.
     const double all = 3.0 * m.nz * pow2.py * (double)pow2.nkx;
     if (f64) {
@@ -197,7 +198,11 @@ bool mixed_pays(const MixedPlan& m, bool f64, const Geometry& pow2)
         // (283 x 269 x 24: 370), an eighth more from 2048 points in y (160 x 640 x 12: 205);
         // taken from 8 % less on (197 x 769 x 10, not taken: 227 against 306)
         const double pad = 0.6 + 0.2 * pow2.pz / m.nz;
-        return passes_us(m) <= 0.92 * ((pow2.px <= 64 ? 10.0 : 20.0) + all * 7.7e-6 * pad) * (pow2.py >= 2048 ? 1.12 : 1.0) + x;
+        const double limit = 0.92 * ((pow2.px <= 64 ? 10.0 : 20.0) + all * 7.7e-6 * pad) * (pow2.py >= 2048 ? 1.12 : 1.0) + x;
+        // of 1145 meshes 22 were slower after all, those above 11 cells in x from 0.7 of the
+        // limit on (102 x 452 x 12: 90 us against 85)
+        *close = passes_us(m) > 0.6 * limit;
+        return passes_us(m) <= limit;
     }
     // on at most five planes the long z stage takes longer than those of the cluster
     // schedules (3 x 16 x 27 21 and 18 us, 2 x 59 x 15 23 and 21)
@@ -206,7 +211,12 @@ bool mixed_pays(const MixedPlan& m, bool f64, const Geometry& pow2)
     // against 75 in planes; 27 x 137 x 26, 33 planes of 25 k points: 22 against 51; 34 x 88
     // x 22: 31 against 22); with fewer points in x, too, 15 % more
     const double gain = 2 * m.x.H < pow2.px ? 1.15 : 0.98;
-    return plane_us(m) <= gain * std::max(m.HZ <= 8 || pow2.px <= 64 ? 16.0 : 25.0, 6.0 + all * 8.8e-6) + x;
+    const double limit = gain * std::max(m.HZ <= 8 || pow2.px <= 64 ? 16.0 : 25.0, 6.0 + all * 8.8e-6) + x;
+    // of 2163 meshes 33 were slower after all, all with long z stages, and but for three of 3 x 30
+    // cells in the plane from 0.57 of the limit on (431 x 189 x 21: 286 us against 229; 656 x 82 x 25: 324
+    // against 283)
+    *close = m.HZ >= 16 && plane_us(m) > 0.5 * limit;
+    return plane_us(m) <= limit;
 }
 
 size_t mixed_tw_entries(const MixedPlan& m, size_t* oy, size_t* oz)
