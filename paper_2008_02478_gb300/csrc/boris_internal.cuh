@@ -50,7 +50,8 @@ struct Geometry {
 struct YZSchedule {
     int kind;     // 0: fused, z stage through shared-memory passes; 1: fused, z stage in
                   // registers; 2: split into y-forward, z-convolution and y-inverse kernels;
-                  // 3: the plane kernel on mixed-radix lengths (mixed_demag.cuh)
+                  // 3, 4: the plane kernel, or y, z and y passes, on mixed-radix lengths
+                  // (mixed_demag.cuh)
     int C;        // kinds 0/1: CTAs per cluster (one cluster per kx plane; ky residues mod C);
                   // kind 2: CTAs per SM targeted by the z-convolution's register budget
     int Qc;       // z-columns processed per chunk of the z stage
@@ -269,7 +270,7 @@ struct PlanView {
     const void* tw;
     bool ml;       // multi-mesh plan
     bool oersted;  // Oersted plan: its spectrum is the curl kernel, not the demag tensor
-    const MixedPlan* mixed;  // mixed-radix path (schedule kind 3), else NULL
+    const MixedPlan* mixed;  // mixed-radix path (schedule kinds 3 and 4), else NULL
     bool mixed_x1024;        // with the power-of-two x passes
 };
 // Number of kernel classes timed by the plan's profiler.

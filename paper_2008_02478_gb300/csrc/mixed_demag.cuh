@@ -1,6 +1,7 @@
-// Convolution on mixed-radix lengths: x passes and the y-z plane kernel
-// (mixed_x.cuh, plane_conv.cuh).  Used by single-mesh FP32 and FP64 plans whose
-// padded kx plane fits one CTA's shared memory.
+// Convolution on mixed-radix lengths: x passes (mixed_x.cuh), and for the y-z part
+// the plane kernel where a padded kx plane fits one CTA's shared memory
+// (plane_conv.cuh; FP32 and FP64) or y, z and y passes (mixed_split.cu; FP32).
+// Single-mesh plans take them by mixed_pays.
 #pragma once
 #include "boris_internal.cuh"
 #include "mixed_fft.cuh"

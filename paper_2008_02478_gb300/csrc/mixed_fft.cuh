@@ -3,8 +3,9 @@
 // The convolution needs a transform length of at least 2n - 1 along an axis of
 // n cells; a power of two wastes up to half of it per axis (n = 160: 512
 // points where 320 suffice).  Here the padded length is 2 H with H >= n from a
-// fine set of products r1 r2 r3 of the radices 2..16 (neighbours within 25 %,
-// most within 20 %), so ragged meshes pay for their own size.
+// fine set of products r1 r2 r3 of the radices 2..16 (from 12 on, a length is at
+// most a third above the one before and on average a fifth; below, up to a half),
+// so ragged meshes pay for their own size.
 //
 // The padded line is zero from n on (n <= H), so its even and odd outputs are
 // two length-H transforms of the same input: X[2k + p] = DFT_H(x[n] w_2H^(p n)).
@@ -83,7 +84,6 @@ void line_tw_host(const LineFFT& f, double2* out);
 void line_pos_host(const LineFFT& f, int esz, unsigned short* out);
 
 // w_N^e (N divides 480) for a compile-time e
-template <int N, typename C> __device__ __forceinline__ C wlit(int e);
 template <int N> struct WLit {
     template <typename C> static __device__ __forceinline__ C get(int e)
     {
