@@ -200,8 +200,9 @@ bool mixed_pays(const MixedPlan& m, bool f64, const Geometry& pow2, bool* close)
         const double pad = 0.6 + 0.2 * pow2.pz / m.nz;
         const double limit = 0.92 * ((pow2.px <= 64 ? 10.0 : 20.0) + all * 7.7e-6 * pad) * (pow2.py >= 2048 ? 1.12 : 1.0) + x;
         // of 1145 meshes 22 were slower after all, those above 11 cells in x from 0.7 of the
-        // limit on (102 x 452 x 12: 90 us against 85)
-        *close = passes_us(m) > 0.6 * limit;
+        // limit on (102 x 452 x 12: 90 us against 85), shorter lines from 0.44 (8 x 394 x 26: 46
+        // against 42)
+        *close = passes_us(m) > (pow2.px <= 32 ? 0.4 : 0.6) * limit;
         return passes_us(m) <= limit;
     }
     // on at most five planes the long z stage takes longer than those of the cluster
